@@ -160,9 +160,10 @@ int fides_ctx_add_stream(fides_ctx *ctx, void *stream);
  * per GPU; every launch here covers all limbs of a step, and what is tuned is
  * the tile width of each pass, which sets the CTA count and hence how full the
  * last wave is).  Times each tile variant (16, 8 or 4 columns or rows per CTA,
- * with a 64- or 80-register budget) of each logN=16 pass for every limb count 1..max_limbs (at most 128; larger
+ * with a 64- or 80-register budget, 16 or 8 elements per thread) of each
+ * two-pass transform's pass for every limb count 1..max_limbs (at most 128; larger
  * launches use the choice for 128) on this context's scratch, and keeps the
- * fastest.  Without it 8 columns / 4 rows per CTA are used.  Results are unchanged
+ * fastest.  Without it the variant goes by the launch's size.  Results are unchanged
  * by the choice.  Synchronises `stream`; do not run it while other work uses
  * this context.  logN = 12 has a single variant (returns FIDES_OK at once).
  * fides_ctx_ntt_tile reports the variant chosen for pass 0..3 (forward

@@ -4,14 +4,16 @@
 // context parameter (Sec. III-F1) whose best value depends on the GPU
 // (Sec. IV).  Here one launch always covers every limb of a step; what is left
 // to tune is the tile width of each pass, which decides how many CTAs a launch
-// has and so how much of its last wave is empty.  Five variants of each pass
-// of a two-pass transform (logN 13..17) are compiled -- at logN=16, 16, 8 or
-// 4 columns/rows per CTA (256, 128 or 64 threads) with up to 80 registers (3,
-// 6 or 12 resident CTAs per SM), and 4 or 8 per CTA with up to 64 registers
-// (16 or 8 per SM); other sizes scale the resident-CTA target to the same
-// register budget (ntt_impl.cuh) -- and the context keeps, per pass kind and
-// limb count, the variant to launch: a fixed default, or the fastest measured
-// one after fides_ctx_autotune.  The launchers of each ring degree live in
+// has and so how much of its last wave is empty, and the elements per thread.
+// Six variants of each pass of a two-pass transform (logN 13..17) are compiled
+// -- at logN=16, sixteen elements per thread with 16, 8 or 4 columns/rows per
+// CTA (256, 128 or 64 threads) and up to 80 registers (3, 6 or 12 resident
+// CTAs per SM), or with 4 or 8 per CTA and up to 64 registers (16 or 8 per
+// SM), and eight elements per thread with 4 per CTA (128 threads, 8 per SM, 64
+// registers); other sizes scale the resident-CTA target to the same register
+// budget (ntt_impl.cuh) -- and the context keeps, per pass kind and limb
+// count, the variant to launch: a default by size, or the fastest measured one
+// after fides_ctx_autotune.  The launchers of each ring degree live in
 // ntt_l12.cu .. ntt_l17.cu; this file dispatches on the context's logN.
 #include <algorithm>
 #include <cstring>
@@ -50,16 +52,31 @@ void tune_one(const fides_ctx *c, int kind, int v, const LimbSet &s, cudaStream_
 }
 }  // namespace
 
-// Default variants before autotuning: 8 columns per CTA for column passes and
-// 4 rows per CTA for row passes (the choice the autotuner makes on GB300 for
-// almost every limb count between 1 and 128).
+// Default variants before autotuning.  A launch of up to 30 limbs at
+// logN = 16 (2 M elements; 6.3 sixteen-element warps per SM sub-partition at
+// most) runs in one wave, whose length is one thread's instruction stream:
+// eight elements per thread halve it and put twice the warps in flight.
+// Larger launches are bound by the multiply pipe, and sixteen elements
+// exchange through shared memory once instead of twice.  Measured in chains of
+// whole transforms (columns + rows, sixteen -> eight elements):
+//   logN = 16 forward:  1 limb 7.7 -> 5.2 us, 10: 20.8 -> 16.1, 20: 22.1 ->
+//     18.2, 30: 25.3 -> 24.8, 36: 28.4 -> 29.6, 90: 62.4 -> 67.2
+//   logN = 16 inverse:  1: 7.8 -> 5.3, 10: 24.1 -> 17.5, 20: 25.8 -> 19.8,
+//     30: 29.4 -> 27.1, 60: 49.7 -> 50.0, 90: 70.5 -> 72.0
+//   logN = 14 forward:  7: 7.7 -> 5.9, 60: 19.7 -> 15.3, 120: 22.9 -> 23.2
+//   logN = 17 forward:  1: 10.0 -> 8.3, 15: 29.5 -> 27.7, 24: 42.2 -> 41.1
+// Above the line, columns run best with 8 per CTA and 64 registers forward
+// (90 limbs: 62.4 -> 60.7 us with 4 rows per CTA at 80 registers), 80
+// registers inverse; inverse rows keep eight elements at every size (90 limbs:
+// the pass alone 1 us faster).
 void ntt_default_variants(fides_ctx *c)
 {
     for (int n = 0; n <= FIDES_TUNE_MAX; ++n) {
-        c->ntt_var[FWD_COLS][n] = 1;
-        c->ntt_var[INV_COLS][n] = 1;
-        c->ntt_var[FWD_ROWS][n] = 2;
-        c->ntt_var[INV_ROWS][n] = 2;
+        const bool one_wave = ((long)n << c->logN) <= (30L << 16);
+        c->ntt_var[FWD_COLS][n] = one_wave ? 5 : 4;
+        c->ntt_var[INV_COLS][n] = one_wave ? 5 : 1;
+        c->ntt_var[FWD_ROWS][n] = one_wave ? 5 : 2;
+        c->ntt_var[INV_ROWS][n] = 5;
     }
 }
 

@@ -6,9 +6,11 @@
 // explicit bit reversal is needed.  Stage s (m = 2^s blocks) of the forward
 // transform pairs j and j + N/2^(s+1) and uses twiddle psi^brv(m + (j >> (logN-s))).
 //
-// Decomposition.  A CTA transforms a tile held in registers (16 elements per
-// thread) and shared memory:
-//   * logN = 12: the whole limb is one tile of 256 threads (KIND 2, one pass);
+// Decomposition.  A CTA transforms a tile held in registers (16 or 8 elements
+// per thread, 2^LE) and shared memory:
+//   * logN = 12: the whole limb is one tile of 512 threads, 8 elements each
+//     (KIND 2, one pass; 15.0 us a launch with 256 threads of 16 elements, 13.3
+//     with 512, three to four limbs, under per-launch events);
 //   * logN = 13..17: two passes as in the paper's hierarchical 2-D NTT -- a
 //     column pass (KIND 0) runs the first S_col stages on CT columns of stride
 //     2^(logN - S_col), a row pass (KIND 1) runs the other S_row stages on CT
@@ -17,25 +19,26 @@
 //     narrower tiles split a small launch into more CTAs so its last wave
 //     costs less (the choice per pass and limb count is autotuned, see
 //     ntt.cu).
-// Inside a pass, stages are grouped four at a time ("rounds"): in a round every
-// thread owns 16 elements whose local indices differ only in the round's four
-// bits, so four radix-2 stages run in registers (a pass whose stage count is
-// not a multiple of four ends with a partial round, see ntt_round); rounds exchange data through
-// shared memory (k-major for columns, XOR-swizzled rows otherwise, both free
-// of bank conflicts).  Loads and stores are coalesced: where the thread-to-
+// Inside a pass, stages are grouped LE at a time ("rounds"): in a round every
+// thread owns 2^LE elements whose local indices differ only in the round's LE
+// bits, so LE radix-2 stages run in registers (a pass whose stage count is
+// not a multiple of LE ends with a partial round, see ntt_round); rounds exchange data through
+// shared memory: k-major for columns, and rows padded by one word in sixteen,
+// whose offsets are immediates (free of bank conflicts with 16 elements per
+// thread, at most two-way with 8).  Loads and stores are coalesced: where the thread-to-
 // element map of the first/last round is strided, the tile is staged through
 // shared memory instead.  The column pass reads its 255 twiddles (shared by
 // every column) from shared memory; the row pass reads per-row twiddles
 // through L1.
 //
-// Twiddle index of a butterfly.  In round rho (bit offset b of the round's four
+// Twiddle index of a butterfly.  In round rho (bit offset b of the round's LE
 // bits in the local index k) the thread's elements are k(r) = X' | r << b | low
-// bits, and the forward stage s = S0 + 4 rho + a of the lower element r uses
-// index 2^s + (X << a) + (r >> (4 - a)); the inverse stage s = S0 + S - 1 -
-// 4 rho - a uses 2^s + (X << (3 - a)) + (r >> (a + 1)).  X collects the bits of
+// bits, and the forward stage s = S0 + LE rho + a of the lower element r uses
+// index 2^s + (X << a) + (r >> (LE - a)); the inverse stage s = S0 + S - 1 -
+// LE rho - a uses 2^s + (X << (LE - 1 - a)) + (r >> (a + 1)).  X collects the bits of
 // the global index above the round's bits (the row for row passes).
 //
-// Arithmetic is lazy (Harvey): forward values stay in [0, 6q) at round
+// Arithmetic is lazy (Harvey): forward values stay in [0, 6q) at pass
 // boundaries and [0, 8q) in between (one conditional subtraction every other
 // stage), inverse values in [0, 2q); primes are below 2^61, so 8q < 2^64.
 // Each butterfly costs one Shoup product, and at most one conditional
@@ -50,17 +53,18 @@
 
 #include "fides_internal.cuh"
 
-// k with its four bits [b, b+3] set to r and the other bits taken from u
+// k with its LE bits [b, b+LE-1] set to r and the other bits taken from u
+template <int LE>
 __device__ __forceinline__ int kmap(int u, int r, int b)
 {
-    return ((u >> b) << (b + 4)) | (r << b) | (u & ((1 << b) - 1));
+    return ((u >> b) << (b + LE)) | (r << b) | (u & ((1 << b) - 1));
 }
 
-// Forward butterfly, reducing x on every other stage only (red): with
-// t = w y in [0, 2q), a reducing stage maps inputs in [0, 8q) to [0, 6q)
-// (x -> csub(x, 4q) in [0, 4q)), a skipping one maps [0, 6q) to [0, 8q);
-// 8q < 2^64 for primes below 2^61, and the Shoup product takes any 64-bit
-// input.  Rounds start and end on [0, 6q).
+// Forward butterfly, reducing x on every other stage only (red), the pass's
+// last stage among them: with t = w y in [0, 2q), a reducing stage maps inputs
+// in [0, 8q) to [0, 6q) (x -> csub(x, 4q) in [0, 4q)), a skipping one maps
+// [0, 6q) to [0, 8q); 8q < 2^64 for primes below 2^61, and the Shoup product
+// takes any 64-bit input.  Passes start and end on [0, 6q).
 // (red is a constant once the stage loop is unrolled)
 __device__ __forceinline__ void ct_bfly(u64 &x, u64 &y, const TwPair &w, u64 q, u64 q2, u64 q4, bool red)
 {
@@ -294,80 +298,83 @@ struct EpiHmRs {
     }
 };
 
-// One round of up to four radix-2 stages on the thread's 16 registers, whose
-// local indices differ in the four bits [B, B+3] (the round's window).  A full
-// round runs the four stages of the window; the last round of a pass whose
-// stage count is not a multiple of four runs only the stages a = A0..3 (its
-// window is the lowest four bits for a forward pass, the highest four for an
+// One round of up to LE radix-2 stages on the thread's 2^LE registers, whose
+// local indices differ in the LE bits [B, B+LE-1] (the round's window).  A full
+// round runs the LE stages of the window; the last round of a pass whose
+// stage count is not a multiple of LE runs only the stages a = A0..LE-1 (its
+// window is the lowest LE bits for a forward pass, the highest LE for an
 // inverse one, and the window bits an earlier round transformed act as
 // independent lanes).  X: the global-index bits above the window; TWS:
 // twiddles come from shared memory instead of global.
 // SCALED: an inverse pass that ends with stage 0 multiplies by the final
 // constant there (gs_bfly_scaled with c, cw = c w1) instead of after it.
-template <bool INV, int S0, int S, int B, int A0, bool TWS, bool SCALED>
-__device__ __forceinline__ void ntt_round(u64 (&x)[16], int X, const TwPair *__restrict__ tw,
+template <int LE, bool INV, int S0, int S, int B, int A0, bool TWS, bool SCALED>
+__device__ __forceinline__ void ntt_round(u64 (&x)[1 << LE], int X, const TwPair *__restrict__ tw,
                                           const TwPair *stw, u64 q, u64 q2, const TwPair &c, const TwPair &cw)
 {
     const u64 q4 = 2 * q2;
 #pragma unroll
-    for (int a = A0; a < 4; ++a) {
-        const int s = INV ? S0 + S - 1 - B - a : S0 + (S - 4 - B) + a;
-        const int h = INV ? (1 << a) : (8 >> a);
-        const int base = (1 << s) + (INV ? (X << (3 - a)) : (X << a));
+    for (int a = A0; a < LE; ++a) {
+        const int st = INV ? S - 1 - B - a : (S - LE - B) + a;   // stage within the pass
+        const int s = S0 + st;
+        const int h = INV ? (1 << a) : ((1 << LE) >> (a + 1));
+        const int base = (1 << s) + (INV ? (X << (LE - 1 - a)) : (X << a));
 #pragma unroll
-        for (int r = 0; r < 16; ++r) {
+        for (int r = 0; r < (1 << LE); ++r) {
             if (r & h) continue;
             if (INV && SCALED && s == 0) {
                 gs_bfly_scaled(x[r], x[r + h], c, cw, q, q2);
                 continue;
             }
-            const int idx = base + (INV ? (r >> (a + 1)) : (r >> (4 - a)));
+            const int idx = base + (INV ? (r >> (a + 1)) : (r >> (LE - a)));
             const TwPair w = TWS ? stw[idx] : tw[idx];
             if (INV) gs_bfly(x[r], x[r + h], w, q, q2);
-            else ct_bfly(x[r], x[r + h], w, q, q2, q4, (a & 1) != 0);   // stages a = 1, 3 reduce
+            else ct_bfly(x[r], x[r + h], w, q, q2, q4, ((S - 1 - st) & 1) == 0);   // the pass's last stage reduces
         }
     }
 }
 
 // Window and first stage of round rho of a pass of S stages (see ntt_round).
-template <int S, bool INV>
+template <int LE, int S, bool INV>
 __host__ __device__ constexpr int round_window(int rho)
 {
-    return (rho == (S + 3) / 4 - 1 && S % 4 != 0) ? (INV ? S - 4 : 0) : (INV ? 4 * rho : S - 4 - 4 * rho);
+    return (rho == (S + LE - 1) / LE - 1 && S % LE != 0) ? (INV ? S - LE : 0) : (INV ? LE * rho : S - LE - LE * rho);
 }
-template <int S>
+template <int LE, int S>
 __host__ __device__ constexpr int round_first(int rho)
 {
-    return (rho == (S + 3) / 4 - 1 && S % 4 != 0) ? 4 - S % 4 : 0;
+    return (rho == (S + LE - 1) / LE - 1 && S % LE != 0) ? LE - S % LE : 0;
 }
 
-// Threads of a tile: 16 elements each.
-template <int S, int KIND, int CT>
+// Threads of a tile: 2^LE elements each.
+template <int S, int KIND, int CT, int LE>
 __host__ __device__ constexpr int ntt_threads()
 {
-    return ((KIND == 2 ? 1 : CT) << S) / 16;
+    return ((KIND == 2 ? 1 : CT) << S) >> LE;
 }
 
 // KIND: 0 = column pass (CT strided columns of 2^S elements, stages 0..S-1),
 //       1 = row pass (CT contiguous rows of 2^S elements, stages LOGN-S..LOGN-1),
-//       2 = whole limb (S == LOGN == 12, 256 threads; CT ignored).
+//       2 = whole limb (S == LOGN == 12; CT ignored).
 // INV selects Gentleman-Sande stages in reverse order; NINV applies N^-1 (or
 // the segment's constant) within the last stage, before the epilogue.  MINB
 // is the resident-CTA target per SM.
-template <int LOGN, int S, int KIND, bool INV, bool NINV, int CT, int MINB, class Pro, class Epi>
-__global__ void __launch_bounds__(ntt_threads<S, KIND, CT>(), MINB)
+template <int LOGN, int S, int KIND, bool INV, bool NINV, int CT, int MINB, int LE, class Pro, class Epi>
+__global__ void __launch_bounds__(ntt_threads<S, KIND, CT, LE>(), MINB)
     k_ntt(LimbSet set, const PrimeInfo *__restrict__ P, const TwPair *__restrict__ TW, Pro pro, Epi epi)
 {
     constexpr int C = (KIND == 2) ? 1 : CT;            // sub-transforms per tile
-    constexpr int THREADS = ntt_threads<S, KIND, CT>();
-    constexpr int RT = (1 << S) / 16;                  // threads per sub-transform
-    constexpr int R = (S + 3) / 4;                     // rounds (the last one may be partial)
+    constexpr int THREADS = ntt_threads<S, KIND, CT, LE>();
+    constexpr int E = 1 << LE;                         // elements per thread
+    constexpr int RT = (1 << S) >> LE;                 // threads per sub-transform
+    constexpr int R = (S + LE - 1) / LE;               // rounds (the last one may be partial)
+    constexpr int RP = (1 << S) + (1 << (S - 4));      // shared-memory words of a padded row
     constexpr int S0 = (KIND == 1) ? (LOGN - S) : 0;
     constexpr int SH = LOGN - S;                       // column stride shift
     constexpr bool TWS = (KIND == 0);                  // column twiddles staged in shared memory
-    static_assert(S >= 5 && R <= 3, "tile shape");
+    static_assert(S >= 5 && R <= 4, "tile shape");
     static_assert(!NINV || (INV && KIND != 1), "the final scale is applied in stage 0, which only this pass holds");
-    __shared__ u64 sm[C << S];
+    __shared__ u64 sm[KIND == 0 ? C << S : C * RP];
     __shared__ TwPair stw[TWS ? (1 << S) : 1];
 
     // the job table, the primes and the twiddles are the context's or the
@@ -397,41 +404,41 @@ __global__ void __launch_bounds__(ntt_threads<S, KIND, CT>(), MINB)
     };
     auto widx = [&](int cc, int k) -> int {
         if (KIND == 0) return k * C + cc;
-        return cc * (1 << S) + (k ^ ((k >> 4) & 15));
+        return cc * RP + k + (k >> 4);
     };
-    // the global-index bits above a round's window of four bits starting at b
-    auto Xof = [&](int b) -> int { return (KIND == 1 ? (cbase << (S - 4 - b)) : 0) | (u >> b); };
+    // the global-index bits above a round's window of LE bits starting at b
+    auto Xof = [&](int b) -> int { return (KIND == 1 ? (cbase << (S - LE - b)) : 0) | (u >> b); };
 
-    u64 x[16];
+    u64 x[E];
 
     // ---------------- load ----------------
     if (!INV || KIND == 0) {
-        const int b0 = INV ? 0 : S - 4;
+        const int b0 = INV ? 0 : S - LE;
 #pragma unroll
-        for (int r = 0; r < 16; ++r) x[r] = pro(J, gidx(cbase, kmap(u, r, b0)), pr);
+        for (int r = 0; r < E; ++r) x[r] = pro(J, gidx(cbase, kmap<LE>(u, r, b0)), pr);
         if (TWS) __syncthreads();
     } else if constexpr (std::is_same<Pro, ProPlain>::value) {
-        // all sixteen loads in flight before the first shared-memory store
-        u64 v[16];
+        // every load in flight before the first shared-memory store
+        u64 v[E];
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
+        for (int i = 0; i < E; ++i) {
             const int e = t + THREADS * i;
             const int cc = e >> S, k = e & ((1 << S) - 1);
             const int cb = (KIND == 2) ? 0 : (int)blockIdx.x * C + cc;
             v[i] = pro(J, gidx(cb, k), pr);
         }
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
+        for (int i = 0; i < E; ++i) {
             const int e = t + THREADS * i;
             sm[widx(e >> S, e & ((1 << S) - 1))] = v[i];
         }
         __syncthreads();
 #pragma unroll
-        for (int r = 0; r < 16; ++r) x[r] = sm[widx(c, kmap(u, r, 0))];
+        for (int r = 0; r < E; ++r) x[r] = sm[widx(c, kmap<LE>(u, r, 0))];
     } else if constexpr (std::is_same<Pro, ProPrep>::value) {
         // four elements' loads in flight before any of them is computed
 #pragma unroll
-        for (int g = 0; g < 16; g += 4) {
+        for (int g = 0; g < E; g += 4) {
             u32 jj[4];
             int ww[4];
             u64 v[4][4];
@@ -449,10 +456,10 @@ __global__ void __launch_bounds__(ntt_threads<S, KIND, CT>(), MINB)
         }
         __syncthreads();
 #pragma unroll
-        for (int r = 0; r < 16; ++r) x[r] = sm[widx(c, kmap(u, r, 0))];
+        for (int r = 0; r < E; ++r) x[r] = sm[widx(c, kmap<LE>(u, r, 0))];
     } else {
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
+        for (int i = 0; i < E; ++i) {
             int e = t + THREADS * i;
             int cc = e >> S, k = e & ((1 << S) - 1);
             int cb = (KIND == 2) ? 0 : (int)blockIdx.x * C + cc;
@@ -460,7 +467,7 @@ __global__ void __launch_bounds__(ntt_threads<S, KIND, CT>(), MINB)
         }
         __syncthreads();
 #pragma unroll
-        for (int r = 0; r < 16; ++r) x[r] = sm[widx(c, kmap(u, r, 0))];
+        for (int r = 0; r < E; ++r) x[r] = sm[widx(c, kmap<LE>(u, r, 0))];
     }
 
     // The final constant of an inverse pass (NINV): N^-1, or the segment's
@@ -481,43 +488,44 @@ __global__ void __launch_bounds__(ntt_threads<S, KIND, CT>(), MINB)
     // ---------------- rounds ----------------
 #define FIDES_NTT_ROUND(RHO)                                                                 \
     if (RHO < R) {                                                                           \
-        constexpr int b = round_window<S, INV>(RHO < R ? RHO : 0);                          \
+        constexpr int b = round_window<LE, S, INV>(RHO < R ? RHO : 0);                          \
         if (RHO > 0) {                                                                       \
-            _Pragma("unroll") for (int r = 0; r < 16; ++r) x[r] = sm[widx(c, kmap(u, r, b))]; \
+            _Pragma("unroll") for (int r = 0; r < E; ++r) x[r] = sm[widx(c, kmap<LE>(u, r, b))]; \
         }                                                                                    \
-        ntt_round<INV, S0, S, b, round_first<S>(RHO < R ? RHO : 0), TWS, NINV>(x, Xof(b), tw, stw, q, q2, nc, nw); \
+        ntt_round<LE, INV, S0, S, b, round_first<LE, S>(RHO < R ? RHO : 0), TWS, NINV>(x, Xof(b), tw, stw, q, q2, nc, nw); \
         if (RHO < R - 1) {                                                                   \
-            _Pragma("unroll") for (int r = 0; r < 16; ++r) sm[widx(c, kmap(u, r, b))] = x[r]; \
+            _Pragma("unroll") for (int r = 0; r < E; ++r) sm[widx(c, kmap<LE>(u, r, b))] = x[r]; \
             __syncthreads();                                                                 \
         }                                                                                    \
     }
     FIDES_NTT_ROUND(0)
     FIDES_NTT_ROUND(1)
     FIDES_NTT_ROUND(2)
+    FIDES_NTT_ROUND(3)
 #undef FIDES_NTT_ROUND
 
     // ---------------- store ----------------
     if (!INV && !Epi::kRaw) {
 #pragma unroll
-        for (int r = 0; r < 16; ++r) x[r] = csub(csub(x[r], 2 * q2), q2);   // [0, 6q) -> [0, 2q)
+        for (int r = 0; r < E; ++r) x[r] = csub(csub(x[r], 2 * q2), q2);   // [0, 6q) -> [0, 2q)
     }
     if (INV || KIND == 0) {
-        const int bl = INV ? S - 4 : 0;
+        const int bl = INV ? S - LE : 0;
 #pragma unroll
-        for (int h = 0; h < 16; h += 8) {
+        for (int h = 0; h < E; h += 8) {
             u64 pa[8], po[8];
 #pragma unroll
-            for (int r = 0; r < 8; ++r) epi.load(J, gidx(cbase, kmap(u, h + r, bl)), pa[r], po[r]);
+            for (int r = 0; r < 8; ++r) epi.load(J, gidx(cbase, kmap<LE>(u, h + r, bl)), pa[r], po[r]);
 #pragma unroll
-            for (int r = 0; r < 8; ++r) epi.store(J, gidx(cbase, kmap(u, h + r, bl)), x[h + r], pa[r], po[r], pr);
+            for (int r = 0; r < 8; ++r) epi.store(J, gidx(cbase, kmap<LE>(u, h + r, bl)), x[h + r], pa[r], po[r], pr);
         }
     } else {
         __syncthreads();   // the last round's shared-memory reads are done
 #pragma unroll
-        for (int r = 0; r < 16; ++r) sm[widx(c, kmap(u, r, 0))] = x[r];
+        for (int r = 0; r < E; ++r) sm[widx(c, kmap<LE>(u, r, 0))] = x[r];
         __syncthreads();
 #pragma unroll
-        for (int h = 0; h < 16; h += 8) {
+        for (int h = 0; h < E; h += 8) {
             u64 pa[8], po[8];
             u32 jj[8];
             int ww[8];

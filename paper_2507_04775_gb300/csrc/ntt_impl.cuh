@@ -8,8 +8,9 @@
 //   logN   13   14   15   16   17
 //   S_col   7    7    8    8    9
 //   S_row   6    7    7    8    8
-// Each pass has five compiled tile variants (columns/rows per CTA and the
-// resident-CTA target, chosen per pass kind and limb count; see ntt.cu).
+// Each pass has six compiled tile variants (columns/rows per CTA, the
+// resident-CTA target and the elements per thread, chosen per pass kind and
+// limb count; see ntt.cu).
 #pragma once
 
 #include <algorithm>
@@ -20,9 +21,14 @@
 
 namespace {
 
-constexpr int NVAR = 5;
-constexpr int VAR_CT[NVAR] = {16, 8, 4, 4, 8};
-constexpr int VAR_MINB[NVAR] = {3, 6, 12, 16, 8};   // at 256-element passes: 3/6/12 up to 80 registers, 16/8 up to 64
+// Tile variants: columns or rows per CTA, resident CTAs per SM at 256-element
+// passes, log2 of the elements per thread.  With sixteen elements 3/6/12 CTAs
+// leave up to 80 registers a thread and 16/8 up to 64; with eight, 8 CTAs of
+// 128 threads leave 64.
+constexpr int NVAR = 6;
+constexpr int VAR_CT[NVAR] = {16, 8, 4, 4, 8, 4};
+constexpr int VAR_MINB[NVAR] = {3, 6, 12, 16, 8, 8};
+constexpr int VAR_LE[NVAR] = {4, 4, 4, 4, 4, 3};
 
 enum PassKind { FWD_COLS = 0, FWD_ROWS = 1, INV_ROWS = 2, INV_COLS = 3 };
 
@@ -44,8 +50,9 @@ struct Split {
 template <int V, int S>
 struct Tile {
     static constexpr int CT = (S >= 9 && VAR_CT[V] > 8) ? 8 : VAR_CT[V];
-    static constexpr int THREADS = (CT << S) / 16;
-    static constexpr int WANT = (16 * VAR_CT[V] * VAR_MINB[V]) / THREADS;
+    static constexpr int LE = VAR_LE[V];
+    static constexpr int THREADS = (CT << S) >> LE;
+    static constexpr int WANT = (((256 * VAR_CT[V]) >> LE) * VAR_MINB[V]) / THREADS;
     static constexpr int MINB = WANT < 1 ? 1 : (WANT > 32 ? 32 : WANT);
 };
 
@@ -55,7 +62,7 @@ void launch_pass(const fides_ctx *c, const LimbSet &set, const TwPair *tw, Pro p
 {
     constexpr int S = KIND == 0 ? Split<LOGN>::COL : Split<LOGN>::ROW;
     using T = Tile<V, S>;
-    auto k = k_ntt<LOGN, S, KIND, INV, NINV, T::CT, T::MINB, Pro, Epi>;
+    auto k = k_ntt<LOGN, S, KIND, INV, NINV, T::CT, T::MINB, T::LE, Pro, Epi>;
     dim3 grid((1 << (LOGN - S)) / T::CT, set.total), block(T::THREADS);
     FIDES_LAUNCH(name, st, k, grid, block, set, (const PrimeInfo *)c->d_prime, tw, pro, epi);
 }
@@ -69,7 +76,8 @@ void launch_pass_v(int v, const fides_ctx *c, const LimbSet &set, const TwPair *
     case 1: launch_pass<LOGN, 1, KIND, INV, NINV>(c, set, tw, pro, epi, st, name); break;
     case 2: launch_pass<LOGN, 2, KIND, INV, NINV>(c, set, tw, pro, epi, st, name); break;
     case 3: launch_pass<LOGN, 3, KIND, INV, NINV>(c, set, tw, pro, epi, st, name); break;
-    default: launch_pass<LOGN, 4, KIND, INV, NINV>(c, set, tw, pro, epi, st, name); break;
+    case 4: launch_pass<LOGN, 4, KIND, INV, NINV>(c, set, tw, pro, epi, st, name); break;
+    default: launch_pass<LOGN, 5, KIND, INV, NINV>(c, set, tw, pro, epi, st, name); break;
     }
 }
 
@@ -78,8 +86,8 @@ int forward(const fides_ctx *c, const LimbSet &set, Pro pro, Epi epi, cudaStream
 {
     if (set.total == 0) return FIDES_OK;
     if constexpr (LOGN == 12) {
-        auto k = k_ntt<12, 12, 2, false, false, 16, 3, Pro, Epi>;
-        FIDES_LAUNCH("k_ntt_fwd_limb", st, k, dim3(1, set.total), dim3(256), set, (const PrimeInfo *)c->d_prime,
+        auto k = k_ntt<12, 12, 2, false, false, 16, 2, 3, Pro, Epi>;
+        FIDES_LAUNCH("k_ntt_fwd_limb", st, k, dim3(1, set.total), dim3(512), set, (const PrimeInfo *)c->d_prime,
                      (const TwPair *)c->d_tw, pro, epi);
     } else {
         launch_pass_v<LOGN, 0, false, false>(variant_of(c, FWD_COLS, set.total), c, set, c->d_tw, pro, EpiLazy{},
@@ -95,8 +103,8 @@ int inverse(const fides_ctx *c, const LimbSet &set, Pro pro, Epi epi, cudaStream
 {
     if (set.total == 0) return FIDES_OK;
     if constexpr (LOGN == 12) {
-        auto k = k_ntt<12, 12, 2, true, true, 16, 3, Pro, Epi>;
-        FIDES_LAUNCH("k_ntt_inv_limb", st, k, dim3(1, set.total), dim3(256), set, (const PrimeInfo *)c->d_prime,
+        auto k = k_ntt<12, 12, 2, true, true, 16, 2, 3, Pro, Epi>;
+        FIDES_LAUNCH("k_ntt_inv_limb", st, k, dim3(1, set.total), dim3(512), set, (const PrimeInfo *)c->d_prime,
                      (const TwPair *)c->d_itw, pro, epi);
     } else {
         launch_pass_v<LOGN, 1, true, false>(variant_of(c, INV_ROWS, set.total), c, set, c->d_itw, pro, EpiLazy{}, st,
