@@ -27,6 +27,7 @@ typedef uint32_t u32;
 #define FIDES_MAX_PRIMES 64
 #define FIDES_MAX_SEG 24
 #define FIDES_MAX_DIGITS 8
+#define FIDES_MAX_HOIST 4    // hoisted rotations that share their launches: two conversion jobs each
 #define FIDES_MAX_STREAMS 16   // streams with their own scratch pool (fides_ctx_add_stream)
 #define FIDES_MAX_SRC 32
 #define FIDES_TUNE_MAX 128   // NTT tile variants are kept per limb count up to this

@@ -447,33 +447,67 @@ int fides_rotate_hoisted_ws(fides_ctx *c, const fides_ct *a, int n_rot, const in
     const size_t S = (size_t)nl * c->N;
     cudaStream_t st = as_stream(stream);
     OpTrace op("op_rotate_hoisted", st);
-    // one ModUp of c1 (the INTT reads c1 itself; the digits' own limbs are c1's)
-    KsBuffers B = ks_buffers(c, a->data + S, nl, nullptr, nullptr, nullptr, 0, 0, carve(c, ws, stream));
+    // One ModUp of c1 (the INTT reads c1 itself; the digits' own limbs are c1's).
+    // The rest runs for up to four rotations at a time, as many as the scratch
+    // pool holds accumulators for, one launch per step: a single rotation's
+    // steps cover 20 to 60 limbs at logN = 16 and are bound by launch latency
+    // and single waves (seven rotations at 15 limbs: 1099 -> 736 us under
+    // per-launch events; eight at a time measured the same as four, and four
+    // fit the conversion's eight inline jobs).
+    // The inverse transform of the special limbs runs in place in the
+    // accumulators, and the converted limbs go to the outputs, which the final
+    // transform overwrites in place, so a rotation takes 2 (nl + K) limbs of
+    // scratch.  Outputs that overlap one another are written one after the
+    // other, through scratch of their own.
+    const Scratch sc = carve(c, ws, stream);
+    KsBuffers B = ks_buffers(c, a->data + S, nl, nullptr, nullptr, nullptr, 0, 0, sc);
+    const size_t N = c->N, ne = (size_t)nl + c->K;
+    bool overlap = false;
+    for (int i = 0; i < n_rot; ++i)
+        for (int k = 0; k < i; ++k) {
+            const uintptr_t x = (uintptr_t)outs[i].data, y = (uintptr_t)outs[k].data, w = 2 * S * sizeof(u64);
+            if (x < y + w && y < x + w) overlap = true;
+        }
+    u64 *pool = sc.dsrc;                         // the whole pool, laid out for this call
+    B.coeff = pool;
+    B.ext = B.coeff + S;
+    u64 *accs = B.ext + (size_t)ks_beta(c, nl) * ne * N;
+    const size_t room = (c->scratch_words - (size_t)(accs - pool)) / (2 * ne * N);
+    int group = overlap ? 1 : (int)std::min<size_t>(room, FIDES_MAX_HOIST);
     if (int rc = run_modup(c, B, st)) return rc;
-    for (int k = 0; k < n_rot; ++k) {
-        B.evk = rks[k];
-        B.out0 = outs[k].data;
-        B.out1 = outs[k].data + S;
-        const u64 g = fides_galois_elt(c, steps[k]);
-        IPArgs ip;
+    for (int k0 = 0; k0 < n_rot; k0 += group) {
+        const int n = std::min(group, n_rot - k0);
+        IPHoistArgs ip;
         memset(&ip, 0, sizeof(ip));
-        ip.one = ks_ip_op(c, B);
-        ip.one.g = g;
-        if (int rc = launch_inner(c, ip, nl + c->K, ks_beta(c, nl), st)) return rc;
-        std::vector<Seg> v;
+        ip.nop = n;
+        std::vector<Seg> inv, fin;
         std::vector<BConvJob> jb;
-        ks_pinv_segs(c, B, v);
-        if (int rc = ntt_inverse(c, inline_set(v), ProSrc{}, EpiCanon{}, st)) return rc;
-        ks_moddown_jobs(c, B, jb);
+        for (int i = 0; i < n; ++i) {
+            const u64 g = fides_galois_elt(c, steps[k0 + i]);
+            B.evk = rks[k0 + i];
+            B.out0 = outs[k0 + i].data;
+            B.out1 = B.out0 + S;
+            B.acc = accs + (size_t)i * 2 * ne * N;
+            B.conv = overlap ? B.acc + 2 * ne * N : B.out0;
+            ip.op[i] = ks_ip_op(c, B);
+            ip.op[i].g = g;
+            for (int t = 0; t < 2; ++t) {
+                u64 *p = B.acc + (t * ne + nl) * N;
+                inv.push_back(seg_of(p, p, c->K, c->L, nullptr, nullptr, 1, 0, c->d_md_nscale));
+                ks_moddown_job(c, p, B.conv + t * S, nl, jb);
+            }
+            ks_final_segs(c, B, fin);
+            Seg &s0 = fin[fin.size() - 2], &s1 = fin.back();
+            s0.mode = 2;                         // out0 = sigma_g(c0) + P^-1 (acc0 - conv0)
+            s0.side = const_cast<u64 *>(a->data);
+            s0.g = g;
+            s1.mode = 0;                         // out1 = P^-1 (acc1 - conv1)
+            outs[k0 + i].scale = a->scale;
+        }
+        if (int rc = launch_inner_hoist(c, ip, nl + c->K, ks_beta(c, nl), st)) return rc;
+        if (int rc = ntt_inverse(c, inline_set(inv), ProSrc{}, EpiCanon{}, st)) return rc;
         if (int rc = launch_bconv(c, inline_bconv(jb), st)) return rc;
-        v.clear();
-        ks_final_segs(c, B, v);
-        v[0].mode = 2;                  // out0 = sigma_g(c0) + P^-1 (acc0 - conv0)
-        v[0].side = const_cast<u64 *>(a->data);
-        v[0].g = g;
-        v[1].mode = 0;                  // out1 = P^-1 (acc1 - conv1)
-        if (int rc = ntt_forward(c, inline_set(v), ProSrc{}, EpiSubMulRot{}, st)) return rc;
-        outs[k].scale = a->scale;
+        if (int rc = ntt_forward(c, inline_set(fin), ProSrc{}, EpiSubMulRot{}, st)) return rc;
     }
     return FIDES_OK;
 }

@@ -132,28 +132,33 @@ inline void ks_pinv_segs(const fides_ctx *c, const KsBuffers &B, std::vector<Seg
                            0, c->d_md_nscale));
 }
 
-// 6. ModDown, base conversion P -> Q_l of both accumulators.
+// 6. ModDown, base conversion P -> Q_l: the K special limbs at pc to the nl
+//    limbs at conv, one job per accumulator.
+inline void ks_moddown_job(const fides_ctx *c, const u64 *pc, u64 *conv, int nl, std::vector<BConvJob> &v)
+{
+    BConvJob J;
+    memset(&J, 0, sizeof(J));
+    J.src = pc;
+    J.n_src = c->K;
+    J.prescaled = 1;
+    J.src_prime0 = c->L;
+    J.scale = c->d_md_scale;
+    J.mat = c->d_md_mat;
+    J.ld = c->L + c->K;
+    J.nrun = 1;
+    J.run[0] = BConvRun{conv, nl, 0};
+    if (c->tc_on & 2) J.tc = (const unsigned char *)c->d_tc + c->tc_md_off;
+    J.tc_corr = 1;
+    J.centred = c->round_nearest;   // round-to-nearest: convert the centred residues
+    J.corr = c->d_md_negp;
+    v.push_back(J);
+}
+
 inline void ks_moddown_jobs(const fides_ctx *c, const KsBuffers &B, std::vector<BConvJob> &v)
 {
     const size_t N = c->N;
-    for (int t = 0; t < 2; ++t) {
-        BConvJob J;
-        memset(&J, 0, sizeof(J));
-        J.src = B.pc + (size_t)t * c->K * N;
-        J.n_src = c->K;
-        J.prescaled = 1;
-        J.src_prime0 = c->L;
-        J.scale = c->d_md_scale;
-        J.mat = c->d_md_mat;
-        J.ld = c->L + c->K;
-        J.nrun = 1;
-        J.run[0] = BConvRun{B.conv + (size_t)t * B.nl * N, B.nl, 0};
-        if (c->tc_on & 2) J.tc = (const unsigned char *)c->d_tc + c->tc_md_off;
-        J.tc_corr = 1;
-        J.centred = c->round_nearest;   // round-to-nearest: convert the centred residues
-        J.corr = c->d_md_negp;
-        v.push_back(J);
-    }
+    for (int t = 0; t < 2; ++t)
+        ks_moddown_job(c, B.pc + (size_t)t * c->K * N, B.conv + (size_t)t * B.nl * N, B.nl, v);
 }
 
 // 7. ModDown, NTT of the converted limbs with the fused epilogue
