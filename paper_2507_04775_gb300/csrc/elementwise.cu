@@ -220,8 +220,57 @@ struct MacArgs {
     int nt, nl, logN, accumulate;
 };
 
+// (k_ptmac and k_cmac.)  The terms stream from HBM once, so that bandwidth
+// bounds the sums; with 128-bit accumulators built from 64-bit products the
+// multiply pipe took longer than the loads (16 constants at 22 limbs of
+// logN = 16: 99 -> 79 us a launch, eight plaintexts at 15 limbs: 48 -> 43 us,
+// 4.4 TB/s).  The terms per step and the CTAs per SM are the fastest of those
+// tried (1 to 16 terms, 1 to 4 CTAs): more terms cost occupancy.
+// The sums of W words over nt terms: load(t, x, y) fetches the terms' words,
+// U terms at a time (every load of them in flight before the first product).
+// Column sums where the prime's size allows (cols_ok), 128-bit ones otherwise.
+template <int W, int U, class Load>
+__device__ __forceinline__ void mac_terms(int nt, const PrimeInfo &p, u64 (&s)[W], Load load)
+{
+    if (cols_ok(nt, p.q)) {
+        AccCols acc[W];
+#pragma unroll
+        for (int i = 0; i < W; ++i) acc[i] = AccCols{s[i], 0, 0, 0};
+        for (int t0 = 0; t0 < nt; t0 += U) {
+            u64 x[U][W], y[U][W];
+#pragma unroll
+            for (int t = 0; t < U; ++t)
+                if (t0 + t < nt) load(t0 + t, x[t], y[t]);
+#pragma unroll
+            for (int t = 0; t < U; ++t)
+                if (t0 + t < nt) {
+#pragma unroll
+                    for (int i = 0; i < W; ++i) mac_cols(acc[i], x[t][i], y[t][i]);
+                }
+        }
+#pragma unroll
+        for (int i = 0; i < W; ++i) {
+            const Acc128 r = cols_sum(acc[i]);
+            s[i] = reduce128(((u64)r.w3 << 32) | r.w2, ((u64)r.w1 << 32) | r.w0, p);
+        }
+        return;
+    }
+    Acc128 acc[W];
+#pragma unroll
+    for (int i = 0; i < W; ++i) acc[i] = Acc128{(u32)s[i], (u32)(s[i] >> 32), 0, 0};
+    for (int t = 0; t < nt; ++t) {
+        u64 x[W], y[W];
+        load(t, x, y);
+#pragma unroll
+        for (int i = 0; i < W; ++i) mac_wide(acc[i], x[i], y[i]);
+    }
+#pragma unroll
+    for (int i = 0; i < W; ++i)
+        s[i] = reduce128(((u64)acc[i].w3 << 32) | acc[i].w2, ((u64)acc[i].w1 << 32) | acc[i].w0, p);
+}
+
 template <bool VEC>
-__global__ void __launch_bounds__(256) k_ptmac(MacArgs A, const PrimeInfo *__restrict__ P)
+__global__ void __launch_bounds__(256, 3) k_ptmac(MacArgs A, const PrimeInfo *__restrict__ P)
 {
     pdl_enter();
     const size_t S = (size_t)A.nl << A.logN;
@@ -230,24 +279,20 @@ __global__ void __launch_bounds__(256) k_ptmac(MacArgs A, const PrimeInfo *__res
     for (size_t v = (size_t)blockIdx.x * blockDim.x + threadIdx.x; v < S / 2; v += (size_t)gridDim.x * blockDim.x) {
         const size_t wi = 2 * v;
         const PrimeInfo p = P[(int)(wi >> A.logN)];
-        U128 s[4] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}};
+        u64 s[4] = {0, 0, 0, 0};
         if (A.accumulate) {
-            load2<VEC>(A.out + wi, s[0].lo, s[1].lo);
-            load2<VEC>(A.out + S + wi, s[2].lo, s[3].lo);
+            load2<VEC>(A.out + wi, s[0], s[1]);
+            load2<VEC>(A.out + S + wi, s[2], s[3]);
         }
-#pragma unroll 2
-        for (int t = 0; t < A.nt; ++t) {
-            u64 x[4], y0, y1;
+        mac_terms<4, 2>(A.nt, p, s, [&](int t, u64 (&x)[4], u64 (&y)[4]) {
             load2<VEC>(A.ct[t] + wi, x[0], x[1]);
             load2<VEC>(A.ct[t] + S + wi, x[2], x[3]);
-            load2<VEC>(A.pt[t] + wi, y0, y1);
-            mac128(s[0], x[0], y0);
-            mac128(s[1], x[1], y1);
-            mac128(s[2], x[2], y0);
-            mac128(s[3], x[3], y1);
-        }
-        store2<VEC>(A.out + wi, reduce128(s[0].hi, s[0].lo, p), reduce128(s[1].hi, s[1].lo, p));
-        store2<VEC>(A.out + S + wi, reduce128(s[2].hi, s[2].lo, p), reduce128(s[3].hi, s[3].lo, p));
+            load2<VEC>(A.pt[t] + wi, y[0], y[1]);
+            y[2] = y[0];
+            y[3] = y[1];
+        });
+        store2<VEC>(A.out + wi, s[0], s[1]);
+        store2<VEC>(A.out + S + wi, s[2], s[3]);
     }
 }
 
@@ -302,7 +347,7 @@ struct CmacArgs {
 };
 
 template <bool VEC>
-__global__ void __launch_bounds__(256) k_cmac(const CmacArgs A, const PrimeInfo *__restrict__ P)
+__global__ void __launch_bounds__(256, 4) k_cmac(const CmacArgs A, const PrimeInfo *__restrict__ P)
 {
     pdl_enter();
     const size_t S = (size_t)A.nl << A.logN;
@@ -313,28 +358,12 @@ __global__ void __launch_bounds__(256) k_cmac(const CmacArgs A, const PrimeInfo 
         const size_t wi = w - (poly ? S : 0);
         const int z = (int)(wi >> A.logN);
         const PrimeInfo p = P[z];
-        U128 s0 = {0, 0}, s1 = {0, 0};
-#pragma unroll 4
-        for (int t = 0; t < A.nt; ++t) {
-            const u64 *src = A.x[t] + (poly ? ((size_t)A.xl[t] << A.logN) + wi : wi);
-            const u64 k = __ldg(A.k + (size_t)A.cidx[t] * A.kld + z);
-            u64 x0, x1;
-            if (VEC) {
-                const ulonglong2 xv = *reinterpret_cast<const ulonglong2 *>(src);
-                x0 = xv.x; x1 = xv.y;
-            } else {
-                x0 = src[0]; x1 = src[1];
-            }
-            mac128(s0, x0, k);
-            mac128(s1, x1, k);
-        }
-        const u64 r0 = reduce128(s0.hi, s0.lo, p), r1 = reduce128(s1.hi, s1.lo, p);
-        if (VEC) {
-            *reinterpret_cast<ulonglong2 *>(A.out + w) = make_ulonglong2(r0, r1);
-        } else {
-            A.out[w] = r0;
-            A.out[w + 1] = r1;
-        }
+        u64 s[2] = {0, 0};
+        mac_terms<2, 4>(A.nt, p, s, [&](int t, u64 (&x)[2], u64 (&y)[2]) {
+            load2<VEC>(A.x[t] + (poly ? ((size_t)A.xl[t] << A.logN) + wi : wi), x[0], x[1]);
+            y[0] = y[1] = __ldg(A.k + (size_t)A.cidx[t] * A.kld + z);
+        });
+        store2<VEC>(A.out + w, s[0], s[1]);
     }
 }
 

@@ -59,29 +59,6 @@ struct BConvArgs {
 
 constexpr int BCONV_TG = 16;     // targets per CTA
 
-struct Acc128 {
-    u32 w0, w1, w2, w3;
-};
-
-// c += a * b for 64-bit a, b (the full 128-bit product), as three carry chains
-// of 32-bit multiply-adds.
-__device__ __forceinline__ void mac_wide(Acc128 &c, u64 a, u64 b)
-{
-    const u32 a0 = (u32)a, a1 = (u32)(a >> 32), b0 = (u32)b, b1 = (u32)(b >> 32);
-    asm("mad.lo.cc.u32 %0, %4, %6, %0;\n\t"
-        "madc.hi.cc.u32 %1, %4, %6, %1;\n\t"
-        "madc.lo.cc.u32 %2, %5, %7, %2;\n\t"
-        "madc.hi.u32 %3, %5, %7, %3;\n\t"
-        "mad.lo.cc.u32 %1, %4, %7, %1;\n\t"
-        "madc.hi.cc.u32 %2, %4, %7, %2;\n\t"
-        "addc.u32 %3, %3, 0;\n\t"
-        "mad.lo.cc.u32 %1, %5, %6, %1;\n\t"
-        "madc.hi.cc.u32 %2, %5, %6, %2;\n\t"
-        "addc.u32 %3, %3, 0;"
-        : "+r"(c.w0), "+r"(c.w1), "+r"(c.w2), "+r"(c.w3)
-        : "r"(a0), "r"(a1), "r"(b0), "r"(b1));
-}
-
 __device__ __forceinline__ u64 reduce_acc(const Acc128 &c, const PrimeInfo &p)
 {
     return reduce128(((u64)c.w3 << 32) | c.w2, ((u64)c.w1 << 32) | c.w0, p);
