@@ -296,6 +296,16 @@ extern "C" void fides_key_destroy(fides_key *k) { free(k); }
 
 extern "C" uint64_t fides_key_galois(const fides_key *k) { return k ? k->g : 0; }
 
+// d of q = 2^k - d, k the bit length of q
+static u64 below_pow2(u64 q) { return ((u64)1 << (64 - __builtin_clzll(q))) - q; }
+
+// whether transforms modulo q can fold (ntt.cuh)
+static bool fold_prime(u64 q)
+{
+    const int k = 64 - __builtin_clzll(q);
+    return k >= 50 && k <= 60 && below_pow2(q) < ((u64)1 << 28);
+}
+
 // fp16 bits of an integer 0 <= k < 256 (exact: at most 8 significant bits).
 static uint16_t f16_of_byte(unsigned k)
 {
@@ -389,6 +399,10 @@ extern "C" int fides_ctx_create(int logN, int L, int dnum, const uint64_t *prime
     c->logN = logN; c->N = N; c->L = L; c->K = K; c->dnum = dnum; c->alpha = alpha;
     memcpy(c->primes, primes, sizeof(u64) * np);
 
+    c->fold = 1;
+    for (int i = 0; i < np; ++i)
+        if (!fold_prime(primes[i])) c->fold = 0;
+
     // per-prime constants and twiddles
     std::vector<PrimeInfo> pinfo(np);
     std::vector<TwPair> tw((size_t)np * N), itw((size_t)np * N);
@@ -407,12 +421,28 @@ extern "C" int fides_ctx_create(int logN, int L, int dnum, const uint64_t *prime
         P.ninvp = shoup_of(P.ninv, q);
         P.ninvw = P.ninvwp = 0;   // after the twiddles
         P.bmu = (u64)(((u128)1 << (63 + (64 - __builtin_clzll(q)))) / q);
+        P.fd2 = P.fsh = 0;
+        P.fbig = P.fK = 0;
+        if (c->fold) {
+            const int k = 64 - __builtin_clzll(q);
+            P.fd2 = (u32)(2 * below_pow2(q));
+            P.fsh = k + 1 - 32;
+            // a folded product is below 2^(k+1) + 2^32 2d; the sums an inverse
+            // butterfly subtracts stay below 2.5 2^61 (k <= 58) or 1.1 2^62
+            const u64 bt = ((u64)2 << k) + ((u64)P.fd2 << 32);
+            P.fbig = (bt / q + 1) * q;
+            P.fK = k <= 58 ? ((u64)3 << 61) / q * q : (((u64)9 << 59) / q + 1) * q;
+        }
+        // a twiddle with its companion: 2^32 w mod q for folding, Shoup's otherwise
+        auto tw_pair = [&](u64 w) {
+            return c->fold ? TwPair{w, (u64)(((u128)w << 32) % q)} : pair_of(w, q);
+        };
         // powers in natural order, then scattered to bit-reversed positions
         u64 x = 1, y = 1;
         for (int k = 0; k < N; ++k) {
             size_t at = (size_t)i * N + bitrev(k, logN);
-            tw[at] = pair_of(x, q);
-            itw[at] = pair_of(y, q);
+            tw[at] = tw_pair(x);
+            itw[at] = tw_pair(y);
             x = hmul(x, psi, q);
             y = hmul(y, ipsi, q);
         }

@@ -51,6 +51,11 @@ struct __align__(16) PrimeInfo {
     u64 ninvw;  // N^-1 w1 mod q, w1 the twiddle of the last inverse stage (psi^-N/2)
     u64 ninvwp; // Shoup companion of ninvw
     u64 bmu;    // floor(2^(63+k) / q), k the bit length of q (reduce_prod)
+    // q = 2^k - d, for transforms that fold at 2^(k+1) (ntt.cuh; zero otherwise)
+    u32 fd2;    // 2d = 2^(k+1) mod q
+    u32 fsh;    // k + 1 - 32
+    u64 fbig;   // multiple of q not below a folded product (forward butterflies)
+    u64 fK;     // multiple of q not below a sum an inverse butterfly subtracts
 };
 
 // One contiguous run of limbs processed by a kernel: limb k of the run reads
@@ -169,6 +174,11 @@ struct fides_ctx {
     int n_spool;
     void *spool_stream[FIDES_MAX_STREAMS];
     u64 *spool[FIDES_MAX_STREAMS];
+
+    // Every prime is 2^k - d with 50 <= k <= 60 and d < 2^28: the twiddle tables
+    // hold (w, 2^32 w mod q) and the transforms fold (ntt.cuh); otherwise the
+    // tables hold (w, Shoup companion).
+    int fold;
 
     // NTT tile variant per pass kind (forward columns, forward rows, inverse
     // rows, inverse columns) and limb count (ntt.cu)

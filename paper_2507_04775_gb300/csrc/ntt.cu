@@ -52,30 +52,32 @@ void tune_one(const fides_ctx *c, int kind, int v, const LimbSet &s, cudaStream_
 }
 }  // namespace
 
-// Default variants before autotuning.  A launch of up to 30 limbs at
-// logN = 16 (2 M elements; 6.3 sixteen-element warps per SM sub-partition at
-// most) runs in one wave, whose length is one thread's instruction stream:
-// eight elements per thread halve it and put twice the warps in flight.
-// Larger launches are bound by the multiply pipe, and sixteen elements
-// exchange through shared memory once instead of twice.  Measured in chains of
-// whole transforms (columns + rows, sixteen -> eight elements):
-//   logN = 16 forward:  1 limb 7.7 -> 5.2 us, 10: 20.8 -> 16.1, 20: 22.1 ->
-//     18.2, 30: 25.3 -> 24.8, 36: 28.4 -> 29.6, 90: 62.4 -> 67.2
-//   logN = 16 inverse:  1: 7.8 -> 5.3, 10: 24.1 -> 17.5, 20: 25.8 -> 19.8,
-//     30: 29.4 -> 27.1, 60: 49.7 -> 50.0, 90: 70.5 -> 72.0
-//   logN = 14 forward:  7: 7.7 -> 5.9, 60: 19.7 -> 15.3, 120: 22.9 -> 23.2
-//   logN = 17 forward:  1: 10.0 -> 8.3, 15: 29.5 -> 27.7, 24: 42.2 -> 41.1
-// Above the line, columns run best with 8 per CTA and 64 registers forward
-// (90 limbs: 62.4 -> 60.7 us with 4 rows per CTA at 80 registers), 80
-// registers inverse; inverse rows keep eight elements at every size (90 limbs:
-// the pass alone 1 us faster).
+// Default variants before autotuning.  A small launch runs in one wave, whose
+// length is one thread's instruction stream: eight elements per thread halve
+// it and put twice the warps in flight.  Larger launches are bound by the
+// multiply pipe and the twiddle reads, and sixteen elements exchange through
+// shared memory once instead of twice.  The column pass crosses over at 22
+// limbs of logN = 16 (1.4 M elements), the forward row pass, whose twiddles
+// come from L2, at 56, and the inverse row pass not within 120.  Chains of
+// whole transforms, columns + rows with sixteen and sixteen elements per
+// thread, eight and eight, sixteen and eight (folding arithmetic, us):
+//   logN = 16 forward  1 limb 6.5 5.0 5.6, 10: 17.5 14.8 12.8, 20: 20.1 15.9
+//     16.6, 24: 20.2 18.8 18.7, 30: 21.9 22.1 20.9, 60: 37.1 40.2 37.2,
+//     90: 53.0 59.1 53.8
+//   logN = 16 inverse  1: 7.3 5.0 6.2, 20: 22.5 17.6 17.6, 30: 25.8 23.7 23.4,
+//     60: 44.4 43.1 41.1, 90: 63.0 62.3 59.2
+//   logN = 17 forward  7: 15.6 15.4 17.7, 12: 21.3 21.1 20.1, 30: 43.6 44.7 43.7
+//   logN = 14 forward  60: 18.7 14.6 15.4, 90: 19.1 17.1 17.0, 120: 20.5 21.4 19.3
+// Forward columns of more than 128 limbs of logN = 16 run best within 64
+// registers (logN = 17, 90 limbs: 123.7 -> 121.7 us; logN = 16, 120 limbs: 71.2
+// -> 72.2).
 void ntt_default_variants(fides_ctx *c)
 {
     for (int n = 0; n <= FIDES_TUNE_MAX; ++n) {
-        const bool one_wave = ((long)n << c->logN) <= (30L << 16);
-        c->ntt_var[FWD_COLS][n] = one_wave ? 5 : 4;
-        c->ntt_var[INV_COLS][n] = one_wave ? 5 : 1;
-        c->ntt_var[FWD_ROWS][n] = one_wave ? 5 : 2;
+        const long elements = (long)n << c->logN;
+        c->ntt_var[FWD_COLS][n] = elements <= (22L << 16) ? 5 : (elements <= (128L << 16) ? 1 : 4);
+        c->ntt_var[INV_COLS][n] = elements <= (22L << 16) ? 5 : 1;
+        c->ntt_var[FWD_ROWS][n] = elements <= (56L << 16) ? 5 : 2;
         c->ntt_var[INV_ROWS][n] = 5;
     }
 }

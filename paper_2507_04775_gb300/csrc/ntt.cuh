@@ -38,7 +38,9 @@
 // LE rho - a uses 2^s + (X << (LE - 1 - a)) + (r >> (a + 1)).  X collects the bits of
 // the global index above the round's bits (the row for row passes).
 //
-// Arithmetic is lazy (Harvey): forward values stay in [0, 6q) at pass
+// Two forms of the butterflies' arithmetic are compiled: folding, for primes
+// just below a power of two, and Shoup products for any others (below).
+// Shoup arithmetic is lazy (Harvey): forward values stay in [0, 6q) at pass
 // boundaries and [0, 8q) in between (one conditional subtraction every other
 // stage), inverse values in [0, 2q); primes are below 2^61, so 8q < 2^64.
 // Each butterfly costs one Shoup product, and at most one conditional
@@ -46,7 +48,7 @@
 // Prologue and epilogue functors let callers fuse element-wise work into the
 // first load and the last store (Sec. III-F5 "Operation Fusions"); epilogues
 // receive values in [0, 2q), except the raw intermediate store of a forward
-// column pass, which keeps [0, 6q) (the row pass accepts it).
+// column pass, which keeps its lazy range (the row pass accepts it).
 #pragma once
 
 #include <type_traits>
@@ -59,6 +61,93 @@ __device__ __forceinline__ int kmap(int u, int r, int b)
 {
     return ((u >> b) << (b + LE)) | (r << b) | (u & ((1 << b) - 1));
 }
+
+// ---- Folding arithmetic, for contexts whose primes are q = 2^k - d with
+// 50 <= k <= 60 and d < 2^28 (fides_ctx::fold), as the walk downward from 2^k of
+// fides_find_primes gives them ----
+//
+// Twiddles come as (w, w' = 2^32 w mod q).  With a = a1 2^32 + a0 the product
+// is T = a0 w + a1 w' < 2^(k+33), and 2^(k+1) = 2d mod q folds its upper part
+// back: t = (T mod 2^(k+1)) + (T >> (k+1)) 2d.  Five 32 x 32 -> 64 multiplies,
+// 20 cycles of a sub-partition's multiply pipe per warp, against six and four
+// half-width ones, 32 cycles, for the Shoup product, whose quotient takes
+// another four.  Butterflies from registers measure 30 cycles against 41.  At
+// logN = 16 a forward column pass of 90 limbs went from 30.4 to 25.8 us, a row
+// pass (which also waits for its twiddles) from 42.4 to 38.6, and HMult at 30
+// limbs from 260.6 to 243.1 us.
+//
+// The price is the range: t < 2^(k+1) + 2^32 2d, up to 1.25 2^61 for k <= 58
+// ("light") and 2^62 for k = 59, 60 ("heavy"), however small q is.  So values
+// are brought below 2^(k+1) + 2^42 by folding x itself (one multiply) where the
+// next additions would leave 64 bits:
+//   forward  a stage adds at most t + q < 1.375 2^61 (1.25 2^62): the operands
+//            that are added to fold at the start of a round of up to four
+//            stages, and again after two stages when heavy;
+//   inverse  sums double: from 2^59 (2^61) three stages reach 5 2^61, and four
+//            stay in range if the two elements that would pass it fold; heavy
+//            ones fold their sums after two stages and after three.  Rounds
+//            end folded.
+struct FoldP {
+    u32 d2, sh, mask;
+    u64 add;       // forward: fbig, inverse: fK
+    bool heavy;
+    __device__ __forceinline__ FoldP(const PrimeInfo &p, bool inv)
+        : d2(p.fd2), sh(p.fsh), mask((1u << p.fsh) - 1), add(inv ? p.fK : p.fbig), heavy(p.fsh > 27)
+    {
+    }
+};
+
+// a w mod q, below 2^(k+1) + 2^32 2d, for any 64-bit a
+__device__ __forceinline__ u64 mul_fold(u64 a, const TwPair &t, const FoldP &p)
+{
+    const u32 a0 = (u32)a, a1 = (u32)(a >> 32);
+    u32 t0, l1, h0, h1;   // T = (h1 h0) 2^32 + t0
+    asm("mul.lo.u32 %0, %4, %6;\n\t"
+        "mul.hi.u32 %1, %4, %6;\n\t"
+        "mul.lo.u32 %2, %4, %7;\n\t"
+        "mul.hi.u32 %3, %4, %7;\n\t"
+        "mad.lo.cc.u32 %2, %5, %9, %2;\n\t"
+        "madc.hi.u32 %3, %5, %9, %3;\n\t"
+        "mad.lo.cc.u32 %0, %5, %8, %0;\n\t"
+        "madc.hi.cc.u32 %1, %5, %8, %1;\n\t"
+        "addc.u32 %3, %3, 0;\n\t"
+        "add.cc.u32 %2, %2, %1;\n\t"
+        "addc.u32 %3, %3, 0;"
+        : "=&r"(t0), "=&r"(l1), "=&r"(h0), "=&r"(h1)
+        : "r"(a0), "r"(a1), "r"((u32)t.w), "r"((u32)(t.w >> 32)), "r"((u32)t.wp), "r"((u32)(t.wp >> 32)));
+    const u32 hi = __funnelshift_r(h0, h1, p.sh);
+    return (((u64)(h0 & p.mask) << 32) | t0) + (u64)hi * p.d2;
+}
+
+// x mod q below 2^(k+1) + 2^(63-k) 2d for any 64-bit x
+__device__ __forceinline__ u64 fold(u64 x, const FoldP &p)
+{
+    const u32 h = (u32)(x >> 32);
+    return (((u64)(h & p.mask) << 32) | (u32)x) + (u64)(h >> p.sh) * p.d2;
+}
+
+// x mod q in [0, 2q) for any 64-bit x: folds at 2^k, below 2^k + 2^(64-k) d
+__device__ __forceinline__ u64 fold_2q(u64 x, const FoldP &p)
+{
+    const u32 h = (u32)(x >> 32);
+    return (((u64)(h & (p.mask >> 1)) << 32) | (u32)x) + (u64)(h >> (p.sh - 1)) * (p.d2 >> 1);
+}
+
+__device__ __forceinline__ void ct_bfly_fold(u64 &x, u64 &y, const TwPair &w, const FoldP &p)
+{
+    const u64 a = x, t = mul_fold(y, w, p);
+    x = a + t;
+    y = a + p.add - t;
+}
+
+__device__ __forceinline__ void gs_bfly_fold(u64 &x, u64 &y, const TwPair &w, const FoldP &p)
+{
+    const u64 a = x, b = y;
+    x = a + b;
+    y = mul_fold(a + p.add - b, w, p);
+}
+
+// ---- Shoup arithmetic, for any primes below 2^61 ----
 
 // Forward butterfly, reducing x on every other stage only (red), the pass's
 // last stage among them: with t = w y in [0, 2q), a reducing stage maps inputs
@@ -85,11 +174,11 @@ __device__ __forceinline__ void gs_bfly(u64 &x, u64 &y, const TwPair &w, u64 q, 
 // The last inverse stage (one twiddle w1) with the final scale c folded in:
 // (x + y) c and (x - y) (w1 c), both in [0, 2q) -- two Shoup products in
 // place of the stage's product, its subtraction and two scalings.
-__device__ __forceinline__ void gs_bfly_scaled(u64 &x, u64 &y, const TwPair &c, const TwPair &cw, u64 q, u64 q2)
+__device__ __forceinline__ void gs_bfly_scaled(u64 &x, u64 &y, const TwPair &c, const TwPair &cw, u64 q, u64 K)
 {
     u64 a = x, b = y;
     x = mul_shoup(a + b, c, q);
-    y = mul_shoup(a + q2 - b, cw, q);
+    y = mul_shoup(a + K - b, cw, q);   // K: a multiple of q not below b
 }
 
 // ---- prologue functors: value of input element j, in [0, 4q) ----
@@ -308,29 +397,59 @@ struct EpiHmRs {
 // twiddles come from shared memory instead of global.
 // SCALED: an inverse pass that ends with stage 0 multiplies by the final
 // constant there (gs_bfly_scaled with c, cw = c w1) instead of after it.
-template <int LE, bool INV, int S0, int S, int B, int A0, bool TWS, bool SCALED>
+// FOLD: the butterflies' arithmetic.  FIRST: the first round of a forward
+// transform, whose inputs need no folding (below 4q).
+template <int LE, bool INV, int S0, int S, int B, int A0, bool TWS, bool SCALED, bool FOLD, bool FIRST>
 __device__ __forceinline__ void ntt_round(u64 (&x)[1 << LE], int X, const TwPair *__restrict__ tw,
-                                          const TwPair *stw, u64 q, u64 q2, const TwPair &c, const TwPair &cw)
+                                          const TwPair *stw, u64 q, u64 q2, const FoldP &fp, const TwPair &c,
+                                          const TwPair &cw)
 {
+    constexpr int E = 1 << LE;
     const u64 q4 = 2 * q2;
 #pragma unroll
     for (int a = A0; a < LE; ++a) {
+        const int n = a - A0;                                    // stages of the round before this one
         const int st = INV ? S - 1 - B - a : (S - LE - B) + a;   // stage within the pass
         const int s = S0 + st;
-        const int h = INV ? (1 << a) : ((1 << LE) >> (a + 1));
+        const int h = INV ? (1 << a) : (E >> (a + 1));
         const int base = (1 << s) + (INV ? (X << (LE - 1 - a)) : (X << a));
+        if (FOLD && !INV && ((n == 0 && !FIRST) || (n == 2 && fp.heavy))) {
 #pragma unroll
-        for (int r = 0; r < (1 << LE); ++r) {
+            for (int r = 0; r < E; ++r)
+                if (!(r & h)) x[r] = fold(x[r], fp);
+        }
+        if (FOLD && INV && n == 2 && fp.heavy) {
+#pragma unroll
+            for (int r = 0; r < E; ++r)
+                if (!(r & (2 << A0))) x[r] = fold(x[r], fp);     // sums of the stage before
+        }
+        if (FOLD && INV && n == 3) {
+            // heavy: products of stage 1, summed in stage 2; light: products of
+            // stage 0, summed in stages 1 and 2
+#pragma unroll
+            for (int r = 0; r < E; ++r) {
+                if (fp.heavy && (r & 2) && !(r & 4)) x[r] = fold(x[r], fp);
+                if (!fp.heavy && (r & 1) && !(r & 6)) x[r] = fold(x[r], fp);
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < E; ++r) {
             if (r & h) continue;
             if (INV && SCALED && s == 0) {
-                gs_bfly_scaled(x[r], x[r + h], c, cw, q, q2);
+                gs_bfly_scaled(x[r], x[r + h], c, cw, q, FOLD ? fp.add : q2);
                 continue;
             }
             const int idx = base + (INV ? (r >> (a + 1)) : (r >> (LE - a)));
             const TwPair w = TWS ? stw[idx] : tw[idx];
-            if (INV) gs_bfly(x[r], x[r + h], w, q, q2);
+            if (FOLD && INV) gs_bfly_fold(x[r], x[r + h], w, fp);
+            else if (FOLD) ct_bfly_fold(x[r], x[r + h], w, fp);
+            else if (INV) gs_bfly(x[r], x[r + h], w, q, q2);
             else ct_bfly(x[r], x[r + h], w, q, q2, q4, ((S - 1 - st) & 1) == 0);   // the pass's last stage reduces
         }
+    }
+    if (FOLD && INV && !(SCALED && B == S - LE)) {
+#pragma unroll
+        for (int r = 0; r < E; ++r) x[r] = fold(x[r], fp);
     }
 }
 
@@ -359,7 +478,7 @@ __host__ __device__ constexpr int ntt_threads()
 // INV selects Gentleman-Sande stages in reverse order; NINV applies N^-1 (or
 // the segment's constant) within the last stage, before the epilogue.  MINB
 // is the resident-CTA target per SM.
-template <int LOGN, int S, int KIND, bool INV, bool NINV, int CT, int MINB, int LE, class Pro, class Epi>
+template <int LOGN, int S, int KIND, bool INV, bool NINV, int CT, int MINB, int LE, bool FOLD, class Pro, class Epi>
 __global__ void __launch_bounds__(ntt_threads<S, KIND, CT, LE>(), MINB)
     k_ntt(LimbSet set, const PrimeInfo *__restrict__ P, const TwPair *__restrict__ TW, Pro pro, Epi epi)
 {
@@ -409,6 +528,7 @@ __global__ void __launch_bounds__(ntt_threads<S, KIND, CT, LE>(), MINB)
     // the global-index bits above a round's window of LE bits starting at b
     auto Xof = [&](int b) -> int { return (KIND == 1 ? (cbase << (S - LE - b)) : 0) | (u >> b); };
 
+    const FoldP fp(pr, INV);
     u64 x[E];
 
     // ---------------- load ----------------
@@ -492,7 +612,8 @@ __global__ void __launch_bounds__(ntt_threads<S, KIND, CT, LE>(), MINB)
         if (RHO > 0) {                                                                       \
             _Pragma("unroll") for (int r = 0; r < E; ++r) x[r] = sm[widx(c, kmap<LE>(u, r, b))]; \
         }                                                                                    \
-        ntt_round<LE, INV, S0, S, b, round_first<LE, S>(RHO < R ? RHO : 0), TWS, NINV>(x, Xof(b), tw, stw, q, q2, nc, nw); \
+        ntt_round<LE, INV, S0, S, b, round_first<LE, S>(RHO < R ? RHO : 0), TWS, NINV, FOLD, RHO == 0 && KIND != 1>( \
+            x, Xof(b), tw, stw, q, q2, fp, nc, nw);                                          \
         if (RHO < R - 1) {                                                                   \
             _Pragma("unroll") for (int r = 0; r < E; ++r) sm[widx(c, kmap<LE>(u, r, b))] = x[r]; \
             __syncthreads();                                                                 \
@@ -507,7 +628,7 @@ __global__ void __launch_bounds__(ntt_threads<S, KIND, CT, LE>(), MINB)
     // ---------------- store ----------------
     if (!INV && !Epi::kRaw) {
 #pragma unroll
-        for (int r = 0; r < E; ++r) x[r] = csub(csub(x[r], 2 * q2), q2);   // [0, 6q) -> [0, 2q)
+        for (int r = 0; r < E; ++r) x[r] = FOLD ? fold_2q(x[r], fp) : csub(csub(x[r], 2 * q2), q2);   // to [0, 2q)
     }
     if (INV || KIND == 0) {
         const int bl = INV ? S - LE : 0;

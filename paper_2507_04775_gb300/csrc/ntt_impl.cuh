@@ -56,13 +56,13 @@ struct Tile {
     static constexpr int MINB = WANT < 1 ? 1 : (WANT > 32 ? 32 : WANT);
 };
 
-template <int LOGN, int V, int KIND, bool INV, bool NINV, class Pro, class Epi>
+template <int LOGN, int V, int KIND, bool INV, bool NINV, bool FOLD, class Pro, class Epi>
 void launch_pass(const fides_ctx *c, const LimbSet &set, const TwPair *tw, Pro pro, Epi epi, cudaStream_t st,
                  const char *name)
 {
     constexpr int S = KIND == 0 ? Split<LOGN>::COL : Split<LOGN>::ROW;
     using T = Tile<V, S>;
-    auto k = k_ntt<LOGN, S, KIND, INV, NINV, T::CT, T::MINB, T::LE, Pro, Epi>;
+    auto k = k_ntt<LOGN, S, KIND, INV, NINV, T::CT, T::MINB, T::LE, FOLD, Pro, Epi>;
     dim3 grid((1 << (LOGN - S)) / T::CT, set.total), block(T::THREADS);
     FIDES_LAUNCH(name, st, k, grid, block, set, (const PrimeInfo *)c->d_prime, tw, pro, epi);
 }
@@ -71,13 +71,25 @@ template <int LOGN, int KIND, bool INV, bool NINV, class Pro, class Epi>
 void launch_pass_v(int v, const fides_ctx *c, const LimbSet &set, const TwPair *tw, Pro pro, Epi epi,
                    cudaStream_t st, const char *name)
 {
+    if (c->fold) {
+        switch (v) {
+        case 0: launch_pass<LOGN, 0, KIND, INV, NINV, true>(c, set, tw, pro, epi, st, name); break;
+        case 1: launch_pass<LOGN, 1, KIND, INV, NINV, true>(c, set, tw, pro, epi, st, name); break;
+        case 2: launch_pass<LOGN, 2, KIND, INV, NINV, true>(c, set, tw, pro, epi, st, name); break;
+        case 3: launch_pass<LOGN, 3, KIND, INV, NINV, true>(c, set, tw, pro, epi, st, name); break;
+        case 4: launch_pass<LOGN, 4, KIND, INV, NINV, true>(c, set, tw, pro, epi, st, name); break;
+        default: launch_pass<LOGN, 5, KIND, INV, NINV, true>(c, set, tw, pro, epi, st, name); break;
+        }
+        return;
+    }
+    // Shoup arithmetic: the wide and the 64-register tiles run as 1 and 2
     switch (v) {
-    case 0: launch_pass<LOGN, 0, KIND, INV, NINV>(c, set, tw, pro, epi, st, name); break;
-    case 1: launch_pass<LOGN, 1, KIND, INV, NINV>(c, set, tw, pro, epi, st, name); break;
-    case 2: launch_pass<LOGN, 2, KIND, INV, NINV>(c, set, tw, pro, epi, st, name); break;
-    case 3: launch_pass<LOGN, 3, KIND, INV, NINV>(c, set, tw, pro, epi, st, name); break;
-    case 4: launch_pass<LOGN, 4, KIND, INV, NINV>(c, set, tw, pro, epi, st, name); break;
-    default: launch_pass<LOGN, 5, KIND, INV, NINV>(c, set, tw, pro, epi, st, name); break;
+    case 0:
+    case 1:
+    case 4: launch_pass<LOGN, 1, KIND, INV, NINV, false>(c, set, tw, pro, epi, st, name); break;
+    case 2:
+    case 3: launch_pass<LOGN, 2, KIND, INV, NINV, false>(c, set, tw, pro, epi, st, name); break;
+    default: launch_pass<LOGN, 5, KIND, INV, NINV, false>(c, set, tw, pro, epi, st, name); break;
     }
 }
 
@@ -86,7 +98,8 @@ int forward(const fides_ctx *c, const LimbSet &set, Pro pro, Epi epi, cudaStream
 {
     if (set.total == 0) return FIDES_OK;
     if constexpr (LOGN == 12) {
-        auto k = k_ntt<12, 12, 2, false, false, 16, 2, 3, Pro, Epi>;
+        auto k = c->fold ? k_ntt<12, 12, 2, false, false, 16, 2, 3, true, Pro, Epi>
+                         : k_ntt<12, 12, 2, false, false, 16, 2, 3, false, Pro, Epi>;
         FIDES_LAUNCH("k_ntt_fwd_limb", st, k, dim3(1, set.total), dim3(512), set, (const PrimeInfo *)c->d_prime,
                      (const TwPair *)c->d_tw, pro, epi);
     } else {
@@ -103,7 +116,8 @@ int inverse(const fides_ctx *c, const LimbSet &set, Pro pro, Epi epi, cudaStream
 {
     if (set.total == 0) return FIDES_OK;
     if constexpr (LOGN == 12) {
-        auto k = k_ntt<12, 12, 2, true, true, 16, 2, 3, Pro, Epi>;
+        auto k = c->fold ? k_ntt<12, 12, 2, true, true, 16, 2, 3, true, Pro, Epi>
+                         : k_ntt<12, 12, 2, true, true, 16, 2, 3, false, Pro, Epi>;
         FIDES_LAUNCH("k_ntt_inv_limb", st, k, dim3(1, set.total), dim3(512), set, (const PrimeInfo *)c->d_prime,
                      (const TwPair *)c->d_itw, pro, epi);
     } else {
