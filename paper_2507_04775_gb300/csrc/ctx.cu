@@ -440,7 +440,9 @@ extern "C" int fides_ctx_create(int logN, int L, int dnum, const uint64_t *prime
         // powers in natural order, then scattered to bit-reversed positions
         u64 x = 1, y = 1;
         for (int k = 0; k < N; ++k) {
-            size_t at = (size_t)i * N + bitrev(k, logN);
+            // psi^k belongs to entry brv(k) = 2^s + i of the bit-reversed order
+            const int e = (int)bitrev(k, logN), st = e ? 31 - __builtin_clz(e) : 0;
+            const size_t at = (size_t)i * N + (e ? tw_index(logN, st, e - (1 << st)) : 0);
             tw[at] = tw_pair(x);
             itw[at] = tw_pair(y);
             x = hmul(x, psi, q);

@@ -112,7 +112,7 @@ struct fides_ctx {
     u64 psi[FIDES_MAX_PRIMES];
 
     PrimeInfo *d_prime;   // [L+K]
-    TwPair *d_tw;         // [L+K][N]   psi^brv(k)
+    TwPair *d_tw;         // [L+K][N]   psi^brv(k) at tw_index (ntt.cuh)
     TwPair *d_itw;        // [L+K][N]   psi^-brv(k)
 
     // ModUp base conversion, per (nl, digit j) at index (nl-1)*dnum + j:

@@ -387,6 +387,20 @@ struct EpiHmRs {
     }
 };
 
+// Table position of twiddle i < 2^s of stage s.  The bit-reversed order keeps
+// entry 2^s + i; the last four stages (a = s - (logN - 4)) are transposed, so
+// that entries i = (X << a) + j of consecutive X are adjacent.  The twiddles of
+// those stages are each thread's own: in the bit-reversed order a row pass's
+// eight loads of the last stage stride 128 bytes across a warp, which took 69 %
+// of the L1's wavefronts; transposed they are 512 contiguous bytes (39 %, a
+// row pass of 90 limbs at logN = 16 35.3 -> 33.5 us, HMult 243.1 -> 239.7).
+__host__ __device__ constexpr int tw_index(int logN, int s, int i)
+{
+    return s < logN - 4 ? (1 << s) + i
+                        : (((1 << (s - logN + 4)) + (i & ((1 << (s - logN + 4)) - 1))) << (logN - 4)) +
+                              (i >> (s - logN + 4));
+}
+
 // One round of up to LE radix-2 stages on the thread's 2^LE registers, whose
 // local indices differ in the LE bits [B, B+LE-1] (the round's window).  A full
 // round runs the LE stages of the window; the last round of a pass whose
@@ -399,7 +413,7 @@ struct EpiHmRs {
 // constant there (gs_bfly_scaled with c, cw = c w1) instead of after it.
 // FOLD: the butterflies' arithmetic.  FIRST: the first round of a forward
 // transform, whose inputs need no folding (below 4q).
-template <int LE, bool INV, int S0, int S, int B, int A0, bool TWS, bool SCALED, bool FOLD, bool FIRST>
+template <int LOGN, int LE, bool INV, int S0, int S, int B, int A0, bool TWS, bool SCALED, bool FOLD, bool FIRST>
 __device__ __forceinline__ void ntt_round(u64 (&x)[1 << LE], int X, const TwPair *__restrict__ tw,
                                           const TwPair *stw, u64 q, u64 q2, const FoldP &fp, const TwPair &c,
                                           const TwPair &cw)
@@ -412,7 +426,7 @@ __device__ __forceinline__ void ntt_round(u64 (&x)[1 << LE], int X, const TwPair
         const int st = INV ? S - 1 - B - a : (S - LE - B) + a;   // stage within the pass
         const int s = S0 + st;
         const int h = INV ? (1 << a) : (E >> (a + 1));
-        const int base = (1 << s) + (INV ? (X << (LE - 1 - a)) : (X << a));
+        const int i0 = INV ? (X << (LE - 1 - a)) : (X << a);
         if (FOLD && !INV && ((n == 0 && !FIRST) || (n == 2 && fp.heavy))) {
 #pragma unroll
             for (int r = 0; r < E; ++r)
@@ -439,8 +453,8 @@ __device__ __forceinline__ void ntt_round(u64 (&x)[1 << LE], int X, const TwPair
                 gs_bfly_scaled(x[r], x[r + h], c, cw, q, FOLD ? fp.add : q2);
                 continue;
             }
-            const int idx = base + (INV ? (r >> (a + 1)) : (r >> (LE - a)));
-            const TwPair w = TWS ? stw[idx] : tw[idx];
+            const int j = INV ? (r >> (a + 1)) : (r >> (LE - a));
+            const TwPair w = TWS ? stw[(1 << s) + i0 + j] : tw[tw_index(LOGN, s, i0 + j)];
             if (FOLD && INV) gs_bfly_fold(x[r], x[r + h], w, fp);
             else if (FOLD) ct_bfly_fold(x[r], x[r + h], w, fp);
             else if (INV) gs_bfly(x[r], x[r + h], w, q, q2);
@@ -612,7 +626,7 @@ __global__ void __launch_bounds__(ntt_threads<S, KIND, CT, LE>(), MINB)
         if (RHO > 0) {                                                                       \
             _Pragma("unroll") for (int r = 0; r < E; ++r) x[r] = sm[widx(c, kmap<LE>(u, r, b))]; \
         }                                                                                    \
-        ntt_round<LE, INV, S0, S, b, round_first<LE, S>(RHO < R ? RHO : 0), TWS, NINV, FOLD, RHO == 0 && KIND != 1>( \
+        ntt_round<LOGN, LE, INV, S0, S, b, round_first<LE, S>(RHO < R ? RHO : 0), TWS, NINV, FOLD, RHO == 0 && KIND != 1>( \
             x, Xof(b), tw, stw, q, q2, fp, nc, nw);                                          \
         if (RHO < R - 1) {                                                                   \
             _Pragma("unroll") for (int r = 0; r < E; ++r) sm[widx(c, kmap<LE>(u, r, b))] = x[r]; \
