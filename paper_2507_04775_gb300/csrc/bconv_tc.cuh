@@ -191,7 +191,12 @@ __device__ __forceinline__ uint4 bytes_f16(u64 x)
     return make_uint4(f16_pair(w0, 0x4140u), f16_pair(w0, 0x4342u), f16_pair(w1, 0x4140u), f16_pair(w1, 0x4342u));
 }
 
+// Forms of the epilogue's reduction (tc_reduce), by the context's primes.
+enum { TC_ANY = 0, TC_BIG = 1, TC_FOLD = 2 };
+
 // Per-target constants of the epilogue.
+// TC_FOLD keeps 2d and, in the upper word, the mask of bits 32..k in p, and
+// k + 1 - 32 in wp.
 struct TcTarget {
     u64 *dst;
     u64 p;
@@ -207,14 +212,26 @@ struct TcTarget {
 // BIG (every target prime >= 2^48): 2^32 mod p = 2^32, and the Shoup quotient
 // floor(hi wp / 2^64) is formed from 32-bit halves without the low x low
 // product, so it may be one too small: hi 2^32 - q p in [0, 3p), and adding
-// lo < p keeps the result below 4p.  Otherwise: full Shoup product and a
-// reduction of lo.
-template <bool BIG>
+// lo < p keeps the result below 4p.  TC_FOLD (primes 2^k - d just below a power
+// of two): V' = sum_k w'_k 2^(16k) < 2^79.7 keeps the exponent bits, which a
+// second element of the offset column (1 against the bytes of minus their sum
+// mod p) takes back, and is folded once at 2^(k+1): (V' mod 2^(k+1)) +
+// (V' >> (k+1)) 2d, below 4p where 2^(k+1) + 2^(78.7-k) 2d is (tc_fold_ok).
+// Thirteen instructions against thirty: the conversions of an HMult at 30 limbs
+// of logN = 16 25.8 -> 23.8 us each, at 36 limbs of logN = 17 60.0 -> 55.0.
+// Otherwise: full Shoup product and a reduction of lo.
+template <int FORM>
 __device__ __forceinline__ u64 tc_reduce(const u32 *r, const TcTarget &T, const PrimeInfo &P)
 {
+    constexpr bool BIG = FORM == TC_BIG;
     u32 w[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) w[k] = r[2 * k + 1] * 256u + r[2 * k];
+    if constexpr (FORM == TC_FOLD) {
+        const u64 lo = (u64)w[1] * 65536u + w[0], h = (u64)w[3] * 65536u + w[2] + (lo >> 32);   // V' = h 2^32 + lo mod 2^32
+        const u32 d2 = (u32)T.p, mask = (u32)(T.p >> 32);
+        return (((u64)((u32)h & mask) << 32) | (u32)lo) + (h >> T.wp) * d2;
+    }
     constexpr u64 OFF = 0x4B000000ull * (1 + (1ull << 16));
     if constexpr (BIG) {
         // 32-bit limbs: lo = (l1, l0), hi = (h1, h0), wp = (v1, v0), p = (p1, p0)
@@ -325,7 +342,7 @@ __device__ __forceinline__ bool pipe_wait(u32 bar, u32 parity, volatile int *abo
 //                         three groups of four warps splitting the targets.
 // So a tile's epilogue overlaps the next tile's MMAs and the bulk copies of
 // the tiles after it.
-template <bool BIG>
+template <int FORM>
 __device__ __forceinline__ void bconv_tc_body(const BConvJob &B, const PrimeInfo *__restrict__ P,
                                               const TwPair *__restrict__ c32, int logN, const TcPipe &pp,
                                               int *status)
@@ -335,7 +352,7 @@ __device__ __forceinline__ void bconv_tc_body(const BConvJob &B, const PrimeInfo
     __shared__ u32 tslot;
     __shared__ volatile int sabort;
     __shared__ TcTarget stg[FIDES_MAX_PRIMES];
-    __shared__ PrimeInfo sp[BIG ? 1 : FIDES_MAX_PRIMES];
+    __shared__ PrimeInfo sp[FORM != TC_ANY ? 1 : FIDES_MAX_PRIMES];
     __shared__ u64 shalf[FIDES_TC_MAX_SRC];
 
     const int t = threadIdx.x, w = t >> 5, lane = t & 31;
@@ -381,19 +398,25 @@ __device__ __forceinline__ void bconv_tc_body(const BConvJob &B, const PrimeInfo
             rem -= B.run[r].count;
         }
         const TwPair cw = c32[pz];
-        stg[t] = TcTarget{ptr, P[pz].q, cw.wp, cw.w};
-        if (!BIG) sp[t] = P[pz];
+        if (FORM == TC_FOLD) {
+            const u32 sh = P[pz].fsh;
+            stg[t] = TcTarget{ptr, ((u64)((1u << sh) - 1) << 32) | P[pz].fd2, sh, 0};
+        } else {
+            stg[t] = TcTarget{ptr, P[pz].q, cw.wp, cw.w};
+        }
+        if (FORM == TC_ANY) sp[t] = P[pz];
     }
     // (q_s - 1) / 2 of the sources (centred jobs; ~0: never above)
     if (t < ns) shalf[t] = B.centred ? (P[B.src_prime0 + t].q >> 1) : ~0ull;
     // constant columns of every A buffer: the offset column (fp16 256 in
-    // element 0 of row m; the image holds 2^15 there for every output byte),
+    // element 0 of row m, where the image holds 2^15 for every output byte, and
+    // 1 in element 1, where it holds TC_FOLD's constant or zero),
     // the correction column (element 0 takes the row's count in centred
     // jobs) and padding
     if (t < TC_M) {
         for (int b = 0; b < pp.na; ++b) {
             unsigned char *arow = sA + b * szA + (t >> 3) * (nsp * 128) + (t & 7) * 16;
-            *(uint4 *)(arow + ns * 128) = make_uint4(0x5C00u, 0, 0, 0);
+            *(uint4 *)(arow + ns * 128) = make_uint4(0x3C005C00u, 0, 0, 0);   // 256, 1
             for (int col = ns + 1; col < nsp; ++col) *(uint4 *)(arow + col * 128) = make_uint4(0, 0, 0, 0);
         }
     }
@@ -505,10 +528,10 @@ __device__ __forceinline__ void bconv_tc_body(const BConvJob &B, const PrimeInfo
                 tc_ld16(acc + 16 * pr, r);
                 const int t0 = 2 * pr;
                 const TcTarget T0 = stg[t0];
-                T0.dst[n] = tc_reduce<BIG>(r, T0, sp[BIG ? 0 : t0]);
+                T0.dst[n] = tc_reduce<FORM>(r, T0, sp[FORM != TC_ANY ? 0 : t0]);
                 if (t0 + 1 < nd) {
                     const TcTarget T1 = stg[t0 + 1];
-                    T1.dst[n] = tc_reduce<BIG>(r + 8, T1, sp[BIG ? 0 : t0 + 1]);
+                    T1.dst[n] = tc_reduce<FORM>(r + 8, T1, sp[FORM != TC_ANY ? 0 : t0 + 1]);
                 }
             }
             tc_fence_before();   // the accumulator's reads are done before it is handed back
@@ -522,7 +545,7 @@ __device__ __forceinline__ void bconv_tc_body(const BConvJob &B, const PrimeInfo
     if (w == 0) tmem_free(tm, pp.ncols);
 }
 
-template <bool BIG>
+template <int FORM>
 __global__ void __launch_bounds__(TC_THREADS, 1) k_bconv_tc(BConvArgs A, const PrimeInfo *__restrict__ P,
                                                             const TwPair *__restrict__ c32, int logN, TcPipe pp,
                                                             int *status)
@@ -530,8 +553,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_bconv_tc(BConvArgs A, const P
     // the dependents may launch now; the body waits for the previous kernel
     // after staging the job's constants
     pdl_trigger();
-    if (A.djob) bconv_tc_body<BIG>(A.djob[blockIdx.y], P, c32, logN, pp, status);
-    else bconv_tc_body<BIG>(A.job[blockIdx.y], P, c32, logN, pp, status);
+    if (A.djob) bconv_tc_body<FORM>(A.djob[blockIdx.y], P, c32, logN, pp, status);
+    else bconv_tc_body<FORM>(A.job[blockIdx.y], P, c32, logN, pp, status);
 }
 
 // Dynamic shared memory of one job with one A buffer and no source stage:
@@ -552,17 +575,17 @@ inline int bconv_tc_smem(const BConvJob &j)
 // conversion shares the SM (it would wait in its allocation).  The source
 // ring is as deep as shared memory allows, up to TC_MAX_DEPTH tiles, with two
 // A buffers, else one.  The CTAs of a job take its N / 128 tiles round robin.
-template <bool BIG>
+template <int FORM>
 inline int launch_bconv_tc_t(const fides_ctx *c, const BConvArgs &G, int max_ns, int max_dst, cudaStream_t st,
                              u64 limit_ns, int stall)
 {
     static int static_smem = -1;
     if (static_smem < 0) {
         cudaFuncAttributes fa;
-        if (cudaFuncGetAttributes(&fa, k_bconv_tc<BIG>) != cudaSuccess)
+        if (cudaFuncGetAttributes(&fa, k_bconv_tc<FORM>) != cudaSuccess)
             return fides_check_cuda(cudaGetLastError(), "bconv tc");
         static_smem = (int)fa.sharedSizeBytes;
-        cudaFuncSetAttribute(k_bconv_tc<BIG>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - static_smem);
+        cudaFuncSetAttribute(k_bconv_tc<FORM>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - static_smem);
     }
     const int ndp = (max_dst + 1) & ~1;
     TcPipe pp;
@@ -610,7 +633,7 @@ inline int launch_bconv_tc_t(const fides_ctx *c, const BConvArgs &G, int max_ns,
         }
     }
     dim3 grid(per_job, G.njob), block(TC_THREADS);
-    FIDES_LAUNCH_SMEM("k_bconv_tc", st, k_bconv_tc<BIG>, grid, block, smem, G, (const PrimeInfo *)c->d_prime,
+    FIDES_LAUNCH_SMEM("k_bconv_tc", st, k_bconv_tc<FORM>, grid, block, smem, G, (const PrimeInfo *)c->d_prime,
                       (const TwPair *)c->d_c32, c->logN, pp, c->d_status);
     return fides_check_cuda(cudaGetLastError(), "bconv tc launch");
 }
@@ -620,8 +643,9 @@ inline int launch_bconv_tc_t(const fides_ctx *c, const BConvArgs &G, int max_ns,
 inline int launch_bconv_tc(const fides_ctx *c, const BConvArgs &G, int max_ns, int max_dst, cudaStream_t st,
                            u64 limit_ns = 2000000000ull, int stall = 0)
 {
-    return c->tc_big ? launch_bconv_tc_t<true>(c, G, max_ns, max_dst, st, limit_ns, stall)
-                     : launch_bconv_tc_t<false>(c, G, max_ns, max_dst, st, limit_ns, stall);
+    return c->tc_form == TC_FOLD ? launch_bconv_tc_t<TC_FOLD>(c, G, max_ns, max_dst, st, limit_ns, stall)
+           : c->tc_form == TC_BIG ? launch_bconv_tc_t<TC_BIG>(c, G, max_ns, max_dst, st, limit_ns, stall)
+                                  : launch_bconv_tc_t<TC_ANY>(c, G, max_ns, max_dst, st, limit_ns, stall);
 }
 
 }  // namespace

@@ -306,6 +306,15 @@ static bool fold_prime(u64 q)
     return k >= 50 && k <= 60 && below_pow2(q) < ((u64)1 << 28);
 }
 
+// whether the conversion's epilogue can fold modulo q (a folding prime): its
+// words make a value below 2^79.7 < 13 2^76, and the folded one must be below 4q
+static bool tc_fold_ok(u64 q)
+{
+    const int k = 64 - __builtin_clzll(q);
+    const u128 folded = ((u128)2 << k) + (((u128)13 << 76) >> (k + 1)) * (2 * below_pow2(q));
+    return folded <= (u128)4 * q;
+}
+
 // fp16 bits of an integer 0 <= k < 256 (exact: at most 8 significant bits).
 static uint16_t f16_of_byte(unsigned k)
 {
@@ -326,7 +335,7 @@ static uint16_t f16_of_byte(unsigned k)
 // with zero blocks.  Returns the image's byte offset.
 template <class F>
 static size_t tc_image(const u64 *primes, const std::vector<int> &targets, int ns, F cst,
-                       std::vector<uint16_t> &img, const u64 *corr = nullptr)
+                       std::vector<uint16_t> &img, bool fold, const u64 *corr = nullptr)
 {
     const size_t off = img.size() * 2;
     const int nd = (int)targets.size(), ndp = (nd + 1) & ~1, nsp = (ns + 2 + (corr ? 1 : 0)) & ~1;
@@ -346,6 +355,14 @@ static size_t tc_image(const u64 *primes, const std::vector<int> &targets, int n
         // offset column: 2^15 (fp16 0x7800) against A's 256 adds 2^23 to every sum
         uint16_t *blk = base + ((size_t)t * nsp + ns) * 64;
         for (int b = 0; b < 8; ++b) blk[b * 8] = 0x7800;
+        // column 1 against A's 1: minus the exponent bits that the folding
+        // epilogue leaves in its words
+        if (fold) {
+            u64 x = 0;
+            for (int k = 0; k < 4; ++k) x = (u64)(((u128)x + (((u128)0x4B000000u << (16 * k)) % p)) % p);
+            x = x ? p - x : 0;
+            for (int b = 0; b < 8; ++b) blk[b * 8 + 1] = f16_of_byte((unsigned)((x >> (8 * b)) & 255));
+        }
         if (corr) {
             uint16_t *cb = base + ((size_t)t * nsp + ns + 1) * 64;
             for (int b = 0; b < 8; ++b)
@@ -507,9 +524,11 @@ extern "C" int fides_ctx_create(int logN, int L, int dnum, const uint64_t *prime
     // [0, L) (a level nl uses the first nl).
     std::vector<uint16_t> tc_img;
     c->tc_on = (alpha <= FIDES_TC_MAX_SRC ? 1 : 0) | (K <= FIDES_TC_MAX_SRC ? 2 : 0);
-    c->tc_big = 1;
-    for (int z = 0; z < np; ++z)
-        if (primes[z] < ((u64)1 << 48)) c->tc_big = 0;
+    c->tc_form = c->fold ? 2 : 1;
+    for (int z = 0; z < np; ++z) {
+        if (c->tc_form == 2 && !tc_fold_ok(primes[z])) c->tc_form = 1;
+        if (primes[z] < ((u64)1 << 48)) c->tc_form = 0;
+    }
     if (c->tc_on & 1) {
         for (int nl = 1; nl <= L; ++nl) {
             int beta = (nl + alpha - 1) / alpha;
@@ -522,7 +541,7 @@ extern "C" int fides_ctx_create(int logN, int L, int dnum, const uint64_t *prime
                 for (int z = L; z < np; ++z) tg.push_back(z);
                 c->tc_mu_off[nl - 1][j] = tc_image(primes, tg, hi - lo,
                                                    [&](int src, int z) { return mu_mat[(off + src) * np + z]; },
-                                                   tc_img);
+                                                   tc_img, c->tc_form == 2);
             }
         }
     }
@@ -530,7 +549,7 @@ extern "C" int fides_ctx_create(int logN, int L, int dnum, const uint64_t *prime
         std::vector<int> tg;
         for (int z = 0; z < L; ++z) tg.push_back(z);
         c->tc_md_off = tc_image(primes, tg, K, [&](int src, int z) { return md_mat[(size_t)src * np + z]; }, tc_img,
-                                md_negp.data());
+                                c->tc_form == 2, md_negp.data());
     }
     if (tc_img.empty()) tc_img.resize(64, 0);
     std::vector<TwPair> c32((size_t)np);

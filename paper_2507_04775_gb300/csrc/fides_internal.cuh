@@ -157,7 +157,7 @@ struct fides_ctx {
     size_t tc_mu_off[FIDES_MAX_PRIMES][FIDES_MAX_DIGITS];
     size_t tc_md_off;
     int tc_on;
-    int tc_big;           // every prime >= 2^48 (the conversion's short epilogue)
+    int tc_form;          // the conversion's epilogue (bconv_tc.cuh): 2 folds, 1 every prime >= 2^48, 0 any
     TwPair *d_c32;
 
     // Device status word: bits set by kernels whose bounded waits ran out

@@ -53,3 +53,31 @@ def test_edges(logN, inside):
 
 def test_mixed_context():
     check(16, [prime_near(16, 54, 1, -1), prime_near(16, 61, 1, -1), prime_near(16, 40, 1, -1)])
+
+
+@pytest.mark.parametrize("k,d", [(50, 1 << 20), (50, 1 << 25), (53, 1 << 26), (53, (1 << 28) - 1), (54, 1),
+                                 (54, (1 << 28) - 1), (59, 1), (60, (1 << 28) - 1)])
+@pytest.mark.parametrize("nearest", [False, True])
+def test_conversions(k, d, nearest):
+    """Key switches whose conversions fold, on both sides of the size of d where
+    they stop (53 bits: between 2^26 and 2^28; 50 bits: 2^20 and 2^25)."""
+    q, step = [], -1 if d == 1 else 1
+    while len(q) < 5:
+        q.append(prime_near(12, k, (1 << k) - q[-1] - 2 * step if q else d, step))
+    p = [prime_near(12, 60, 1, -1)]
+    while len(p) < 2 or p[-1] in q:
+        p.append(prime_near(12, 60, (1 << 60) - p[-1] + 2, -1))
+    p = [x for x in p if x not in q][:2]
+    g, o = Context(12, q, p, 2), oracle.Context(12, q, p, 2)
+    assert g.tensor_bconv
+    g.set_rounding(nearest)
+    o.set_rounding(nearest)
+    st = si.Stream(1950 + k)
+    a = np.stack([si.uniform_poly(st, q, o.N) for _ in range(2)])
+    b = np.stack([si.uniform_poly(st, q, o.N) for _ in range(2)])
+    a[:, :, ::5] = np.array(q, dtype=np.uint64)[:, None] - 1
+    key = np.stack([np.stack([si.uniform_poly(st, o.primes, o.N) for _ in range(2)]) for _ in range(2)])
+    out = torch.empty_like(to_device(a))
+    g.hmult(to_device(a), to_device(b), 5, g.relin_key(to_device(key)), out)
+    assert np.array_equal(to_host(out).reshape(a.shape), o.hmult(a, b, key))
+    g.close()
