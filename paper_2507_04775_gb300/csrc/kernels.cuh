@@ -11,6 +11,7 @@
 
 #include "fides_internal.cuh"
 #include "ntt.cuh"
+#include "rows_inner.cuh"
 
 namespace {
 
@@ -58,30 +59,6 @@ struct BConvArgs {
 };
 
 constexpr int BCONV_TG = 16;     // targets per CTA
-
-__device__ __forceinline__ u64 reduce_acc(const Acc128 &c, const PrimeInfo &p)
-{
-    return reduce128(((u64)c.w3 << 32) | c.w2, ((u64)c.w1 << 32) | c.w0, p);
-}
-
-// the same for a sum of at most two products of canonical residues
-__device__ __forceinline__ u64 reduce_acc2(const Acc128 &c, const PrimeInfo &p)
-{
-    return csub(csub(reduce_prod(((u64)c.w3 << 32) | c.w2, ((u64)c.w1 << 32) | c.w0, p), p.q2), p.q);
-}
-
-// The same for a sum of m products of canonical residues: the Barrett form
-// where its bound holds, m q^2 < 2^(k+63) for m at most 2^(63-k) (k the bit
-// length of q: m <= 4 at 61-bit primes, 8 at 60-bit), reduce128 otherwise.
-__device__ __forceinline__ bool reduce_prod_ok(int m, const PrimeInfo &p)
-{
-    return (u64)m <= (1ull << (__clzll((long long)p.q) - 1));   // 2^(63-k), k = 64 - clz(q)
-}
-__device__ __forceinline__ u64 reduce_accm(const Acc128 &c, const PrimeInfo &p, bool barrett)
-{
-    const u64 hi = ((u64)c.w3 << 32) | c.w2, lo = ((u64)c.w1 << 32) | c.w0;
-    return barrett ? csub(csub(reduce_prod(hi, lo, p), p.q2), p.q) : reduce128(hi, lo, p);
-}
 
 template <int NS>
 __device__ __forceinline__ void bconv_body(const BConvJob &B, const PrimeInfo *__restrict__ P, int logN, int tg)
@@ -288,27 +265,6 @@ inline int launch_bconv(const fides_ctx *c, const BConvArgs &A, cudaStream_t st)
 // d~_j[z] is the ModUp output ext_j[z], except on the limbs of digit j itself,
 // where it is the key-switch input d[z] (read from dsrc, no copy is made).
 // ---------------------------------------------------------------------------
-struct IPOp {
-    const u64 *ext;     // [beta][ne][N]
-    const u64 *dsrc;    // [nl][N] evaluation-form input
-    const u64 *evk;     // [dnum][2][L+K][N]
-    u64 *acc;           // [2][ne][N]
-    int nl, ne, beta, alpha;
-    u64 g;              // 0, or the Galois element through which the digits are read (hoisted rotation)
-};
-
-// One op inline (dop == nullptr; grid.y = its ne limbs) or a device table of
-// ops with a row table: row r (grid.y) computes limb drow[r] & 127 of op
-// drow[r] >> 7 (an op has at most FIDES_MAX_PRIMES limbs).  The batched path orders the rows by key and key limb, so
-// that the ops sharing a key (every HMult of a batch shares the
-// relinearisation key) read each key limb while it is in L2.
-struct IPArgs {
-    const IPOp *dop;
-    const int *drow;
-    int nop;
-    IPOp one;
-};
-
 // Hoisted rotations of one ciphertext, inline: grid.y = nop x their ne limbs,
 // the rotations' rows of one limb next to each other, so that the digits they
 // share come from L2.

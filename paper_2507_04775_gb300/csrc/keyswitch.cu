@@ -55,33 +55,80 @@ __global__ void __launch_bounds__(256) k_hr_last(const u64 *lastc, const u64 *co
     last[(size_t)t * N + n] = csub(csub(x, p.q2), p.q);
 }
 
-int run_modup(const fides_ctx *c, const KsBuffers &B, cudaStream_t st)
+// ModUp up to the converted digits in coefficient form (ext); `extra`: segments
+// transformed along with its input
+int run_modup_conv(const fides_ctx *c, const KsBuffers &B, const std::vector<Seg> &extra, cudaStream_t st)
 {
     std::vector<Seg> v;
     std::vector<BConvJob> jb;
     ks_intt_segs(c, B, v);
+    v.insert(v.end(), extra.begin(), extra.end());
     if (int rc = ntt_inverse(c, inline_set(v), ProSrc{}, EpiCanon{}, st)) return rc;
     ks_modup_jobs(c, B, jb);
-    if (int rc = launch_bconv(c, inline_bconv(jb), st)) return rc;
-    v.clear();
+    return launch_bconv(c, inline_bconv(jb), st);
+}
+
+int run_modup(const fides_ctx *c, const KsBuffers &B, cudaStream_t st)
+{
+    if (int rc = run_modup_conv(c, B, {}, st)) return rc;
+    std::vector<Seg> v;
     ks_modup_ntt_segs(c, B, v);
     return ntt_forward(c, inline_set(v), ProSrc{}, EpiCanon{}, st);
 }
 
-int run_keyswitch(const fides_ctx *c, const KsBuffers &B, cudaStream_t st)
+// Limb l of an HMult fused with Rescale, which the key switch's inverse
+// transforms take along: d (one limb of each polynomial of the tensor product)
+// to dst[0], dst[1], the accumulators to dst[2], dst[3], N words each.
+struct DroppedLimb {
+    const u64 *d0, *d1;
+    u64 *dst;
+    int l;
+};
+
+// Key switch up to the coefficient form of the special limbs of both
+// accumulators (pc, scaled for the ModDown conversion); the q-limbs of the
+// accumulators are in acc.
+int run_ks_front(const fides_ctx *c, const KsBuffers &B, const DroppedLimb *x, cudaStream_t st)
 {
-    if (int rc = run_modup(c, B, st)) return rc;
+    const size_t N = c->N, ne = (size_t)B.nl + c->K;
     IPArgs ip;
     memset(&ip, 0, sizeof(ip));
     ip.one = ks_ip_op(c, B);
-    if (int rc = launch_inner(c, ip, B.nl + c->K, ks_beta(c, B.nl), st)) return rc;
+    std::vector<Seg> v, extra;
+    if (x) {
+        extra.push_back(seg_of(x->d0, x->dst, 1, x->l));
+        extra.push_back(seg_of(x->d1, x->dst + N, 1, x->l));
+    }
+    // (a tensor product fused into the first inverse pass has no d0, d1 yet)
+    if (rows_inner_ok(c, ip.one.beta, B.nl + c->K) && !(x && B.prep)) {
+        if (int rc = run_modup_conv(c, B, extra, st)) return rc;
+        ks_modup_ntt_segs(c, B, v);
+        if (int rc = ntt_fwd_cols(c, inline_set(v), st)) return rc;
+        v.clear();
+        ks_pcols_segs(c, B, v);
+        if (x) {
+            ip.one.xdst = x->dst + 2 * N;
+            ip.one.xl = x->l;
+            for (int t = 2; t < 4; ++t) v.push_back(seg_of(x->dst + t * N, x->dst + t * N, 1, x->l));
+        }
+        if (int rc = ntt_rows_inner(c, ip, B.nl + c->K, ip.one.beta, st)) return rc;
+        return ntt_inv_cols(c, inline_set(v), st);
+    }
+    if (int rc = run_modup(c, B, st)) return rc;
+    if (int rc = launch_inner(c, ip, B.nl + c->K, ip.one.beta, st)) return rc;
+    ks_pinv_segs(c, B, v);
+    v.insert(v.end(), extra.begin(), extra.end());
+    for (int t = 0; x && t < 2; ++t) v.push_back(seg_of(B.acc + (t * ne + x->l) * N, x->dst + (2 + t) * N, 1, x->l));
+    return ntt_inverse(c, inline_set(v), ProSrc{}, EpiCanon{}, st);
+}
+
+int run_keyswitch(const fides_ctx *c, const KsBuffers &B, cudaStream_t st)
+{
+    if (int rc = run_ks_front(c, B, nullptr, st)) return rc;
     std::vector<Seg> v;
     std::vector<BConvJob> jb;
-    ks_pinv_segs(c, B, v);
-    if (int rc = ntt_inverse(c, inline_set(v), ProSrc{}, EpiCanon{}, st)) return rc;
     ks_moddown_jobs(c, B, jb);
     if (int rc = launch_bconv(c, inline_bconv(jb), st)) return rc;
-    v.clear();
     ks_final_segs(c, B, v);
     return ntt_forward(c, inline_set(v), ProSrc{}, EpiSubMul{}, st);
 }
@@ -325,18 +372,11 @@ int fides_hmult_rescale_ws(fides_ctx *c, const fides_ct *a, const fides_ct *b, c
         B.pb = b->data;
         B.pout = sc.dd;
     }
-    if (int rc = run_modup(c, B, st)) return rc;
-    IPArgs ip;
-    memset(&ip, 0, sizeof(ip));
-    ip.one = ks_ip_op(c, B);
-    if (int rc = launch_inner(c, ip, nl + c->K, ks_beta(c, nl), st)) return rc;
-    // ModDown INTT of the special limbs, plus limb l of d0, d1, acc0, acc1
+    // limb l of d0, d1 and of the accumulators goes through the inverse
+    // transforms of the key switch
+    const DroppedLimb x = {sc.dd + (size_t)l * N, sc.dd + S + (size_t)l * N, sc.lastc, l};
+    if (int rc = run_ks_front(c, B, &x, st)) return rc;
     std::vector<Seg> v;
-    ks_pinv_segs(c, B, v);
-    for (int t = 0; t < 2; ++t) v.push_back(seg_of(sc.dd + t * S + (size_t)l * N, sc.lastc + t * N, 1, l));
-    for (int t = 0; t < 2; ++t)
-        v.push_back(seg_of(B.acc + (t * ne + l) * N, sc.lastc + (2 + t) * N, 1, l));
-    if (int rc = ntt_inverse(c, inline_set(v), ProSrc{}, EpiCanon{}, st)) return rc;
     std::vector<BConvJob> jb;
     ks_moddown_jobs(c, B, jb);
     if (int rc = launch_bconv(c, inline_bconv(jb), st)) return rc;

@@ -14,17 +14,18 @@
 
 namespace {
 
-enum LaunchKind { L_INTT, L_BCONV, L_NTT, L_INNER, L_NTT_SUBMUL, L_NTT_SWITCH_SUBMUL, L_TENSOR };
+enum LaunchKind { L_INTT, L_BCONV, L_NTT, L_INNER, L_NTT_SUBMUL, L_NTT_SWITCH_SUBMUL, L_TENSOR,
+                  L_FWD_COLS, L_ROWS_INNER, L_INV_COLS };
 
 struct Launch {
     LaunchKind kind;
     LimbSet set;       // NTT kinds (device segments)
     BConvArgs bc;      // L_BCONV (device jobs)
     int ns, max_dst;
-    IPArgs ip;         // L_INNER
-    int max_beta;      // L_INNER
+    IPArgs ip;         // L_INNER, L_ROWS_INNER
+    int max_beta;      // L_INNER, L_ROWS_INNER
     int ip_pairs;      // L_INNER: every op can take the paired path
-    int total;         // grid.y of L_INNER and L_TENSOR
+    int total;         // grid.y of L_INNER, L_ROWS_INNER and L_TENSOR
     TensorArgs tp;     // L_TENSOR (device ops)
 };
 
@@ -119,19 +120,20 @@ void plan_bconv(Plan &P, const std::vector<BConvJob> &jobs)
     }
 }
 
-void plan_inner(Plan &P, const std::vector<IPOp> &ops, const std::vector<int> &rows)
+void plan_inner(Plan &P, const std::vector<IPOp> &ops, const std::vector<int> &rows, LaunchKind kind)
 {
     if (ops.empty()) return;
     Launch l;
     memset(&l, 0, sizeof(l));
-    l.kind = L_INNER;
+    l.kind = kind;
     // rows (op, limb) ordered by key, then by the key limb the row reads,
-    // then by op: the ops sharing a key read each of its limbs back to back
+    // then by op: the ops sharing a key read each of its limbs back to back.
+    // The special limbs come first: k_rows_inner has most work there.
     struct Row { const u64 *evk; int pz, op, z; };
     std::vector<Row> order;
     for (size_t i = 0; i < ops.size(); ++i)
         for (int z = 0; z < rows[i]; ++z)
-            order.push_back(Row{ops[i].evk, z < ops[i].nl ? z : 1024 + (z - ops[i].nl), (int)i, z});
+            order.push_back(Row{ops[i].evk, z < ops[i].nl ? 1024 + z : z - ops[i].nl, (int)i, z});
     std::stable_sort(order.begin(), order.end(), [](const Row &a, const Row &b) {
         if (a.evk != b.evk) return a.evk < b.evk;
         return a.pz < b.pz;
@@ -216,11 +218,14 @@ void plan_stage(const fides_ctx *c, fides_op *ops, int n_ops, int stage, u64 *co
                 bool tensor_split = true, bool prime_major = false)
 {
     const size_t N = c->N;
-    std::vector<Seg> intt, ntt, pinv, fin, rsfin;
+    std::vector<Seg> intt, ntt, pinv, fin, rsfin, fcols, pcols;
     std::vector<BConvJob> up, down;
-    std::vector<IPOp> ip;
-    std::vector<int> ip_rows;
+    std::vector<IPOp> ip, ri;
+    std::vector<int> ip_rows, ri_rows;
     std::vector<TensorOp> tens;
+    int stage_limbs = 0;   // extended limbs of the stage's key switches
+    for (int i = 0; i < n_ops; ++i)
+        if (ops[i].stage == stage && ops[i].type != FIDES_OP_RESCALE) stage_limbs += ops[i].a.n_limbs + c->K;
     for (int i = 0; i < n_ops; ++i) {
         fides_op &o = ops[i];
         if (o.stage != stage) continue;
@@ -252,10 +257,17 @@ void plan_stage(const fides_ctx *c, fides_op *ops, int n_ops, int stage, u64 *co
         ks_carve(c, B, dsrc + S);
         ks_intt_segs(c, B, intt);
         ks_modup_jobs(c, B, up);
-        ks_modup_ntt_segs(c, B, ntt);
-        ip.push_back(ks_ip_op(c, B));
-        ip_rows.push_back(nl + c->K);
-        ks_pinv_segs(c, B, pinv);
+        if (rows_inner_ok(c, ks_beta(c, nl), stage_limbs)) {
+            ks_modup_ntt_segs(c, B, fcols);
+            ri.push_back(ks_ip_op(c, B));
+            ri_rows.push_back(nl + c->K);
+            ks_pcols_segs(c, B, pcols);
+        } else {
+            ks_modup_ntt_segs(c, B, ntt);
+            ip.push_back(ks_ip_op(c, B));
+            ip_rows.push_back(nl + c->K);
+            ks_pinv_segs(c, B, pinv);
+        }
         ks_moddown_jobs(c, B, down);
         ks_final_segs(c, B, fin);
         o.out.scale = hm ? o.a.scale * o.b.scale : o.a.scale;
@@ -264,8 +276,11 @@ void plan_stage(const fides_ctx *c, fides_op *ops, int n_ops, int stage, u64 *co
     plan_ntt(P, L_INTT, intt, N, prime_major);
     plan_bconv(P, up);
     plan_ntt(P, L_NTT, ntt, N, prime_major);
-    plan_inner(P, ip, ip_rows);
+    plan_inner(P, ip, ip_rows, L_INNER);
     plan_ntt(P, L_INTT, pinv, N, prime_major);
+    plan_ntt(P, L_FWD_COLS, fcols, N, prime_major);
+    plan_inner(P, ri, ri_rows, L_ROWS_INNER);
+    plan_ntt(P, L_INV_COLS, pcols, N, prime_major);
     plan_bconv(P, down);
     plan_ntt(P, L_NTT_SUBMUL, fin, N, prime_major);
     plan_ntt(P, L_NTT_SWITCH_SUBMUL, rsfin, N, prime_major);
@@ -299,6 +314,9 @@ int plan_run(const fides_ctx *c, const std::vector<Launch> &launches, cudaStream
         case L_NTT_SUBMUL: rc = ntt_forward(c, l.set, ProSrc{}, EpiSubMul{}, st); break;
         case L_NTT_SWITCH_SUBMUL: rc = ntt_forward(c, l.set, ProSwitchMod{}, EpiSubMul{}, st); break;
         case L_BCONV: rc = launch_bconv_group(c, l.bc, l.ns, l.max_dst, st); break;
+        case L_FWD_COLS: rc = ntt_fwd_cols(c, l.set, st); break;
+        case L_ROWS_INNER: rc = ntt_rows_inner(c, l.ip, l.total, l.max_beta, st); break;
+        case L_INV_COLS: rc = ntt_inv_cols(c, l.set, st); break;
         case L_INNER: rc = launch_inner(c, l.ip, l.total, l.max_beta, st, l.ip_pairs); break;
         case L_TENSOR: rc = launch_tensor_args(c, l.tp, l.total, st); break;
         }

@@ -44,6 +44,12 @@ int ntt_fwd_submul_rot(const fides_ctx *c, const LimbSet &s, cudaStream_t st)
 int ntt_fwd_raise(const fides_ctx *c, const LimbSet &s, cudaStream_t st) { FIDES_NTT_DISPATCH(ntt_fwd_raise, c, s, st) }
 int ntt_fwd_hmrs(const fides_ctx *c, const LimbSet &s, cudaStream_t st) { FIDES_NTT_DISPATCH(ntt_fwd_hmrs, c, s, st) }
 int ntt_inv_canon(const fides_ctx *c, const LimbSet &s, cudaStream_t st) { FIDES_NTT_DISPATCH(ntt_inv_canon, c, s, st) }
+int ntt_fwd_cols(const fides_ctx *c, const LimbSet &s, cudaStream_t st) { FIDES_NTT_DISPATCH(ntt_fwd_cols, c, s, st) }
+int ntt_inv_cols(const fides_ctx *c, const LimbSet &s, cudaStream_t st) { FIDES_NTT_DISPATCH(ntt_inv_cols, c, s, st) }
+int ntt_rows_inner(const fides_ctx *c, const IPArgs &A, int limbs, int max_beta, cudaStream_t st)
+{
+    FIDES_NTT_DISPATCH(ntt_rows_inner, c, A, limbs, max_beta, st)
+}
 
 namespace {
 void tune_one(const fides_ctx *c, int kind, int v, const LimbSet &s, cudaStream_t st)

@@ -412,9 +412,11 @@ __host__ __device__ constexpr int tw_index(int logN, int s, int i)
 // SCALED: an inverse pass that ends with stage 0 multiplies by the final
 // constant there (gs_bfly_scaled with c, cw = c w1) instead of after it.
 // FOLD: the butterflies' arithmetic.  FIRST: the first round of a forward
-// transform, whose inputs need no folding (below 4q).
-template <int LOGN, int LE, bool INV, int S0, int S, int B, int A0, bool TWS, bool SCALED, bool FOLD, bool FIRST>
-__device__ __forceinline__ void ntt_round(u64 (&x)[1 << LE], int X, const TwPair *__restrict__ tw,
+// transform, whose inputs need no folding (below 4q).  ND: transforms under
+// the same prime side by side, which share each twiddle.
+#define FIDES_ND _Pragma("unroll") for (int d = 0; d < ND; ++d)
+template <int LOGN, int ND, int LE, bool INV, int S0, int S, int B, int A0, bool TWS, bool SCALED, bool FOLD, bool FIRST>
+__device__ __forceinline__ void ntt_round(u64 (&x)[ND][1 << LE], int X, const TwPair *__restrict__ tw,
                                           const TwPair *stw, u64 q, u64 q2, const FoldP &fp, const TwPair &c,
                                           const TwPair &cw)
 {
@@ -430,42 +432,45 @@ __device__ __forceinline__ void ntt_round(u64 (&x)[1 << LE], int X, const TwPair
         if (FOLD && !INV && ((n == 0 && !FIRST) || (n == 2 && fp.heavy))) {
 #pragma unroll
             for (int r = 0; r < E; ++r)
-                if (!(r & h)) x[r] = fold(x[r], fp);
+                if (!(r & h)) FIDES_ND x[d][r] = fold(x[d][r], fp);
         }
         if (FOLD && INV && n == 2 && fp.heavy) {
 #pragma unroll
             for (int r = 0; r < E; ++r)
-                if (!(r & (2 << A0))) x[r] = fold(x[r], fp);     // sums of the stage before
+                if (!(r & (2 << A0))) FIDES_ND x[d][r] = fold(x[d][r], fp);     // sums of the stage before
         }
         if (FOLD && INV && n == 3) {
             // heavy: products of stage 1, summed in stage 2; light: products of
             // stage 0, summed in stages 1 and 2
 #pragma unroll
             for (int r = 0; r < E; ++r) {
-                if (fp.heavy && (r & 2) && !(r & 4)) x[r] = fold(x[r], fp);
-                if (!fp.heavy && (r & 1) && !(r & 6)) x[r] = fold(x[r], fp);
+                if (fp.heavy && (r & 2) && !(r & 4)) FIDES_ND x[d][r] = fold(x[d][r], fp);
+                if (!fp.heavy && (r & 1) && !(r & 6)) FIDES_ND x[d][r] = fold(x[d][r], fp);
             }
         }
 #pragma unroll
         for (int r = 0; r < E; ++r) {
             if (r & h) continue;
             if (INV && SCALED && s == 0) {
-                gs_bfly_scaled(x[r], x[r + h], c, cw, q, FOLD ? fp.add : q2);
+                FIDES_ND gs_bfly_scaled(x[d][r], x[d][r + h], c, cw, q, FOLD ? fp.add : q2);
                 continue;
             }
             const int j = INV ? (r >> (a + 1)) : (r >> (LE - a));
             const TwPair w = TWS ? stw[(1 << s) + i0 + j] : tw[tw_index(LOGN, s, i0 + j)];
-            if (FOLD && INV) gs_bfly_fold(x[r], x[r + h], w, fp);
-            else if (FOLD) ct_bfly_fold(x[r], x[r + h], w, fp);
-            else if (INV) gs_bfly(x[r], x[r + h], w, q, q2);
-            else ct_bfly(x[r], x[r + h], w, q, q2, q4, ((S - 1 - st) & 1) == 0);   // the pass's last stage reduces
+            FIDES_ND {
+                if (FOLD && INV) gs_bfly_fold(x[d][r], x[d][r + h], w, fp);
+                else if (FOLD) ct_bfly_fold(x[d][r], x[d][r + h], w, fp);
+                else if (INV) gs_bfly(x[d][r], x[d][r + h], w, q, q2);
+                else ct_bfly(x[d][r], x[d][r + h], w, q, q2, q4, ((S - 1 - st) & 1) == 0);   // the last stage reduces
+            }
         }
     }
     if (FOLD && INV && !(SCALED && B == S - LE)) {
 #pragma unroll
-        for (int r = 0; r < E; ++r) x[r] = fold(x[r], fp);
+        for (int r = 0; r < E; ++r) FIDES_ND x[d][r] = fold(x[d][r], fp);
     }
 }
+#undef FIDES_ND
 
 // Window and first stage of round rho of a pass of S stages (see ntt_round).
 template <int LE, int S, bool INV>
@@ -543,7 +548,8 @@ __global__ void __launch_bounds__(ntt_threads<S, KIND, CT, LE>(), MINB)
     auto Xof = [&](int b) -> int { return (KIND == 1 ? (cbase << (S - LE - b)) : 0) | (u >> b); };
 
     const FoldP fp(pr, INV);
-    u64 x[E];
+    u64 xd[1][E];
+    u64 (&x)[E] = xd[0];
 
     // ---------------- load ----------------
     if (!INV || KIND == 0) {
@@ -626,8 +632,8 @@ __global__ void __launch_bounds__(ntt_threads<S, KIND, CT, LE>(), MINB)
         if (RHO > 0) {                                                                       \
             _Pragma("unroll") for (int r = 0; r < E; ++r) x[r] = sm[widx(c, kmap<LE>(u, r, b))]; \
         }                                                                                    \
-        ntt_round<LOGN, LE, INV, S0, S, b, round_first<LE, S>(RHO < R ? RHO : 0), TWS, NINV, FOLD, RHO == 0 && KIND != 1>( \
-            x, Xof(b), tw, stw, q, q2, fp, nc, nw);                                          \
+        ntt_round<LOGN, 1, LE, INV, S0, S, b, round_first<LE, S>(RHO < R ? RHO : 0), TWS, NINV, FOLD, RHO == 0 && KIND != 1>( \
+            xd, Xof(b), tw, stw, q, q2, fp, nc, nw);                                          \
         if (RHO < R - 1) {                                                                   \
             _Pragma("unroll") for (int r = 0; r < E; ++r) sm[widx(c, kmap<LE>(u, r, b))] = x[r]; \
             __syncthreads();                                                                 \
@@ -691,6 +697,10 @@ int ntt_fwd_submul_rot(const fides_ctx *c, const LimbSet &set, cudaStream_t st);
 int ntt_fwd_raise(const fides_ctx *c, const LimbSet &set, cudaStream_t st);           // ProRaise, EpiCanon
 int ntt_fwd_hmrs(const fides_ctx *c, const LimbSet &set, cudaStream_t st);            // ProHmRs, EpiHmRs
 int ntt_inv_canon(const fides_ctx *c, const LimbSet &set, cudaStream_t st);           // ProPrep (ProPlain), EpiCanon
+// One pass of a two-pass transform, for callers that fuse the other one
+// (rows_inner.cuh); logN = 12 has no column pass (nothing is launched).
+int ntt_fwd_cols(const fides_ctx *c, const LimbSet &set, cudaStream_t st);            // ProSrc, raw intermediate in dst
+int ntt_inv_cols(const fides_ctx *c, const LimbSet &set, cudaStream_t st);            // from dst, EpiCanon
 
 inline int ntt_forward(const fides_ctx *c, const LimbSet &s, ProSrc, EpiCanon, cudaStream_t st)
 {

@@ -18,6 +18,7 @@
 
 #include "fides_internal.cuh"
 #include "ntt.cuh"
+#include "rows_inner.cuh"
 
 namespace {
 
@@ -129,6 +130,57 @@ int inverse(const fides_ctx *c, const LimbSet &set, Pro pro, Epi epi, cudaStream
     return fides_check_cuda(cudaGetLastError(), "ntt inverse launch");
 }
 
+// the column pass alone (see ntt.cuh)
+template <int LOGN>
+int forward_cols(const fides_ctx *c, const LimbSet &set, cudaStream_t st)
+{
+    if constexpr (LOGN != 12) {
+        if (set.total == 0) return FIDES_OK;
+        launch_pass_v<LOGN, 0, false, false>(variant_of(c, FWD_COLS, set.total), c, set, c->d_tw, ProSrc{}, EpiLazy{},
+                                             st, "k_ntt_fwd_cols");
+    }
+    return fides_check_cuda(cudaGetLastError(), "ntt forward launch");
+}
+
+template <int LOGN>
+int inverse_cols(const fides_ctx *c, const LimbSet &set, cudaStream_t st)
+{
+    if constexpr (LOGN != 12) {
+        if (set.total == 0) return FIDES_OK;
+        launch_pass_v<LOGN, 0, true, true>(variant_of(c, INV_COLS, set.total), c, set, c->d_itw, ProDst{}, EpiCanon{},
+                                           st, "k_ntt_inv_cols");
+    }
+    return fides_check_cuda(cudaGetLastError(), "ntt inverse launch");
+}
+
+// the forward row pass of ModUp's limbs with the key inner product
+// (rows_inner.cuh)
+template <int LOGN, int MAXB>
+int rows_inner_b(const fides_ctx *c, const IPArgs &A, int limbs, int max_beta, cudaStream_t st)
+{
+    constexpr int S = Split<LOGN>::ROW;
+    constexpr int C = 1024 >> S;
+    const dim3 grid((1 << (LOGN - S)) / C, limbs), block((C << S) >> RI_LE);
+    FIDES_LAUNCH_SMEM("k_rows_inner", st, (k_rows_inner<LOGN, S, C, MAXB>), grid, block, rows_inner_smem(max_beta), A,
+                      c->L, c->K, (const PrimeInfo *)c->d_prime, (const TwPair *)c->d_tw, (const TwPair *)c->d_itw);
+    return fides_check_cuda(cudaGetLastError(), "rows + inner product launch");
+}
+
+template <int LOGN>
+int rows_inner(const fides_ctx *c, const IPArgs &A, int limbs, int max_beta, cudaStream_t st)
+{
+    if constexpr (LOGN != 12) {
+        switch (max_beta) {
+        case 1:
+        case 2: return rows_inner_b<LOGN, 2>(c, A, limbs, max_beta, st);
+        case 3: return rows_inner_b<LOGN, 3>(c, A, limbs, max_beta, st);
+        case 4: return rows_inner_b<LOGN, 4>(c, A, limbs, max_beta, st);
+        default: return rows_inner_b<LOGN, 5>(c, A, limbs, max_beta, st);
+        }
+    }
+    return fides_set_error(FIDES_ERR_UNSUPPORTED, "rows + inner product: logN = 12");   // rows_inner_ok is false
+}
+
 // one pass of kind `kind` with variant v (for the autotuner)
 template <int LOGN>
 void launch_one(const fides_ctx *c, int kind, int v, const LimbSet &set, cudaStream_t st)
@@ -160,6 +212,9 @@ void launch_one(const fides_ctx *c, int kind, int v, const LimbSet &set, cudaStr
     int ntt_fwd_raise_##L(const fides_ctx *, const LimbSet &, cudaStream_t);                      \
     int ntt_fwd_hmrs_##L(const fides_ctx *, const LimbSet &, cudaStream_t);                       \
     int ntt_inv_canon_##L(const fides_ctx *, const LimbSet &, cudaStream_t);                      \
+    int ntt_fwd_cols_##L(const fides_ctx *, const LimbSet &, cudaStream_t);                       \
+    int ntt_inv_cols_##L(const fides_ctx *, const LimbSet &, cudaStream_t);                       \
+    int ntt_rows_inner_##L(const fides_ctx *, const IPArgs &, int, int, cudaStream_t);            \
     void ntt_tune_one_##L(const fides_ctx *, int, int, const LimbSet &, cudaStream_t);
 
 #define FIDES_NTT_DEGREE(L)                                                                                       \
@@ -191,6 +246,12 @@ void launch_one(const fides_ctx *c, int kind, int v, const LimbSet &set, cudaStr
     {                                                                                                             \
         if (s.modes == 0) return inverse<L>(c, s, ProPlain{}, EpiCanon{}, st);                                    \
         return inverse<L>(c, s, ProPrep{c->logN}, EpiCanon{}, st);                                                \
+    }                                                                                                             \
+    int ntt_fwd_cols_##L(const fides_ctx *c, const LimbSet &s, cudaStream_t st) { return forward_cols<L>(c, s, st); } \
+    int ntt_inv_cols_##L(const fides_ctx *c, const LimbSet &s, cudaStream_t st) { return inverse_cols<L>(c, s, st); } \
+    int ntt_rows_inner_##L(const fides_ctx *c, const IPArgs &A, int limbs, int max_beta, cudaStream_t st)       \
+    {                                                                                                             \
+        return rows_inner<L>(c, A, limbs, max_beta, st);                                                          \
     }                                                                                                             \
     void ntt_tune_one_##L(const fides_ctx *c, int kind, int v, const LimbSet &s, cudaStream_t st)               \
     {                                                                                                             \

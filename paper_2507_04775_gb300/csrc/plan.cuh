@@ -120,7 +120,21 @@ inline IPOp ks_ip_op(const fides_ctx *c, const KsBuffers &B)
     o.ext = B.ext; o.dsrc = B.d; o.evk = B.evk; o.acc = B.acc;
     o.nl = B.nl; o.ne = B.nl + c->K; o.beta = ks_beta(c, B.nl); o.alpha = c->alpha;
     o.g = 0;
+    o.pc = B.pc;
+    o.xdst = nullptr;
+    o.xl = -1;
     return o;
+}
+
+// Steps 3 to 5 with k_rows_inner: the forward column pass of the converted
+// limbs (ks_modup_ntt_segs), the row pass with the inner product and the
+// inverse row pass of the special limbs, then the inverse column pass of those.
+inline void ks_pcols_segs(const fides_ctx *c, const KsBuffers &B, std::vector<Seg> &v)
+{
+    for (int t = 0; t < 2; ++t) {
+        u64 *p = B.pc + (size_t)t * c->K * c->N;
+        v.push_back(seg_of(p, p, c->K, c->L, nullptr, nullptr, 1, 0, c->d_md_nscale));
+    }
 }
 
 // 5. ModDown, INTT of both accumulators' special limbs.
