@@ -25,7 +25,8 @@ namespace {
 // (Sec. III-F3: lazy 128-bit accumulation, one reduction before the
 // write-back).  The conversion matrix of the group is staged in shared memory
 // (every thread reads the same entry).  NS is the exact number of source limbs
-// (0: any number up to FIDES_MAX_SRC, with guarded loops).
+// (0: any number up to FIDES_MAX_SRC, with guarded loops), or with RAG the
+// largest of the launch (a job's missing sources count as zeros).
 // ---------------------------------------------------------------------------
 struct BConvRun {
     u64 *dst;
@@ -53,6 +54,7 @@ struct BConvJob {
 struct BConvArgs {
     int njob;
     int tc;                  // 1: every job has a tensor-core image (k_bconv_tc)
+    int ragged;              // integer kernel: the jobs' source counts differ
     int tc_smem;             // k_bconv_tc: dynamic shared memory of the largest job (bconv_tc_smem)
     const BConvJob *djob;
     BConvJob job[FIDES_MAX_DIGITS];
@@ -60,7 +62,7 @@ struct BConvArgs {
 
 constexpr int BCONV_TG = 16;     // targets per CTA
 
-template <int NS>
+template <int NS, bool RAG>
 __device__ __forceinline__ void bconv_body(const BConvJob &B, const PrimeInfo *__restrict__ P, int logN, int tg)
 {
     constexpr int MS = NS > 0 ? NS : FIDES_MAX_SRC;
@@ -69,7 +71,8 @@ __device__ __forceinline__ void bconv_body(const BConvJob &B, const PrimeInfo *_
     __shared__ u64 *sdst[BCONV_TG];
     __shared__ u64 scorr[BCONV_TG];
     const int N = 1 << logN;
-    const int ns = NS > 0 ? NS : B.n_src;
+    const int ns = NS > 0 && !RAG ? NS : B.n_src;
+    constexpr bool FULL = NS > 0 && !RAG;   // every job has NS sources
 
     int ndst = 0;
     for (int r = 0; r < B.nrun; ++r) ndst += B.run[r].count;
@@ -91,7 +94,12 @@ __device__ __forceinline__ void bconv_body(const BConvJob &B, const PrimeInfo *_
         sdst[threadIdx.x] = ptr;
         scorr[threadIdx.x] = B.centred ? B.corr[pz] : 0;
         for (int i = 0; i < ns; ++i) smat[threadIdx.x * MS + i] = B.mat[(size_t)i * B.ld + pz];
+        if (RAG)
+            for (int i = ns; i < MS; ++i) smat[threadIdx.x * MS + i] = 0;
     }
+    // all of the above is the host's or the context's; the sources are the
+    // previous kernel's
+    pdl_wait();
     __syncthreads();
 
     const int n = blockIdx.x * blockDim.x + threadIdx.x;
@@ -99,7 +107,7 @@ __device__ __forceinline__ void bconv_body(const BConvJob &B, const PrimeInfo *_
     u64 v[MS];
 #pragma unroll
     for (int i = 0; i < MS; ++i) {
-        if (NS > 0 || i < ns) {
+        if (FULL || i < ns) {
             const u64 x = src[(size_t)i * N + n];
             if (B.prescaled) {
                 v[i] = x;
@@ -117,7 +125,7 @@ __device__ __forceinline__ void bconv_body(const BConvJob &B, const PrimeInfo *_
     if (B.centred) {
 #pragma unroll
         for (int i = 0; i < MS; ++i)
-            if (NS > 0 || i < ns) cnt += v[i] > (P[B.src_prime0 + i].q >> 1) ? 1 : 0;
+            if (FULL || i < ns) cnt += v[i] > (P[B.src_prime0 + i].q >> 1) ? 1 : 0;
     }
     int d = 0;
     for (; d + 1 < nd; d += 2) {
@@ -148,12 +156,12 @@ __device__ __forceinline__ void bconv_body(const BConvJob &B, const PrimeInfo *_
     }
 }
 
-template <int NS>
+template <int NS, bool RAG>
 __global__ void __launch_bounds__(256) k_bconv(BConvArgs A, const PrimeInfo *__restrict__ P, int logN, int tg)
 {
-    pdl_enter();
-    if (A.djob) bconv_body<NS>(A.djob[blockIdx.y], P, logN, tg);
-    else bconv_body<NS>(A.job[blockIdx.y], P, logN, tg);
+    pdl_trigger();   // the body waits after staging the job's constants
+    if (A.djob) bconv_body<NS, RAG>(A.djob[blockIdx.y], P, logN, tg);
+    else bconv_body<NS, RAG>(A.job[blockIdx.y], P, logN, tg);
 }
 
 // Targets per CTA: the group size minimising (waves of CTAs) x (per-CTA time),
@@ -179,12 +187,12 @@ inline int bconv_group(const fides_ctx *c, int njob, int max_dst)
     return best;
 }
 
-template <int NS>
+template <int NS, bool RAG = false>
 void launch_bconv_ns(const fides_ctx *c, const BConvArgs &A, int max_dst, cudaStream_t st)
 {
     const int tg = bconv_group(c, A.njob, max_dst);
     dim3 grid(c->N / 256, A.njob, (max_dst + tg - 1) / tg), block(256);
-    FIDES_LAUNCH("k_bconv", st, k_bconv<NS>, grid, block, A, c->d_prime, c->logN, tg);
+    FIDES_LAUNCH("k_bconv", st, (k_bconv<NS, RAG>), grid, block, A, c->d_prime, c->logN, tg);
 }
 
 }  // namespace
@@ -198,6 +206,12 @@ namespace {
 inline int launch_bconv_group(const fides_ctx *c, const BConvArgs &G, int ns, int max_dst, cudaStream_t st)
 {
     if (G.tc) return launch_bconv_tc(c, G, ns, max_dst, st);
+    if (G.ragged) {
+        if (ns <= 4) launch_bconv_ns<4, true>(c, G, max_dst, st);
+        else if (ns <= 8) launch_bconv_ns<8, true>(c, G, max_dst, st);
+        else launch_bconv_ns<12, true>(c, G, max_dst, st);
+        return fides_check_cuda(cudaGetLastError(), "bconv launch");
+    }
     switch (ns) {
     case 1: launch_bconv_ns<1>(c, G, max_dst, st); break;
     case 2: launch_bconv_ns<2>(c, G, max_dst, st); break;
@@ -223,6 +237,44 @@ inline int bconv_targets(const BConvJob &j)
     return nd;
 }
 
+// Whether the launch's jobs are so small that the integer kernel is faster, in
+// one launch whatever their source counts.  The tensor-core kernel's set-up
+// (barriers, tensor memory, the matrix image, four roles to fill) takes longer
+// than few products, and its time per tile hardly depends on the targets, while
+// the integer kernel's grows with them: up to ten targets and 2^22 products in
+// all, or six and 2^24, of at most twelve sources (at logN = 12, where the
+// tensor-core kernel has one tile per CTA, up to four targets).  HMult by integer
+// against tensor-core conversions, us: logN = 16, 10 special primes, 1 limb 57.9
+// 78.7, 4 limbs 71.0 83.3, 6: 85.6 89.6, 8 (10.5 M products in ModDown) 92.3
+// 92.0; logN = 17, 4 + 9 limbs 111.3 121.6; logN = 15, 7 + 7 limbs 53.8 66.1,
+// 14 + 7 (14 targets, 6.4 M) 88.3 82.3; logN = 14, 10 + 10 limbs 52.7 59.1, 7 + 3
+// 51.2 56.5; logN = 13, 12 + 5 limbs (15 targets, 1.2 M) 52.4 51.6; logN = 12,
+// 4 + 4 limbs 34.4 41.6, 6 + 4 (8 targets) 45.0 40.3.
+template <class V>
+inline bool bconv_small(const fides_ctx *c, const V &jobs, int n)
+{
+    long work = 0;
+    int nd = 0;
+    for (int j = 0; j < n; ++j) {
+        if (jobs[j].n_src > 12) return false;
+        work += (long)jobs[j].n_src * bconv_targets(jobs[j]);
+        nd = std::max(nd, bconv_targets(jobs[j]));
+    }
+    return nd <= (c->logN == 12 ? 4 : 10) && (work << c->logN) <= (nd <= 6 ? 1L << 24 : 1L << 22);
+}
+
+// One integer launch for the jobs, of at most twelve sources each: the largest
+// source count, and whether they differ.
+template <class V>
+inline int bconv_sources(const V &jobs, int n, int *ragged)
+{
+    int ns = 0;
+    for (int j = 0; j < n; ++j) ns = std::max(ns, jobs[j].n_src);
+    *ragged = 0;
+    for (int j = 0; j < n; ++j) *ragged |= jobs[j].n_src != ns;
+    return ns;
+}
+
 // Launch group of a job: every job with a tensor-core image goes to one
 // k_bconv_tc launch (-1); the integer kernel gets one launch per distinct
 // source count (a ragged last digit gets its own, so every launch runs fully
@@ -237,6 +289,13 @@ inline int bconv_group_key(const BConvJob &j)
 inline int launch_bconv(const fides_ctx *c, const BConvArgs &A, cudaStream_t st)
 {
     if (A.njob == 0) return FIDES_OK;
+    if (bconv_small(c, A.job, A.njob)) {
+        BConvArgs G = A;
+        const int ns = bconv_sources(A.job, A.njob, &G.ragged);
+        int max_dst = 0;
+        for (int j = 0; j < A.njob; ++j) max_dst = std::max(max_dst, bconv_targets(A.job[j]));
+        return launch_bconv_group(c, G, ns, max_dst, st);
+    }
     bool done[FIDES_MAX_DIGITS] = {false};
     for (int j = 0; j < A.njob; ++j) {
         if (done[j]) continue;

@@ -91,16 +91,17 @@ inline int plan_bconv_key(const BConvJob &j)
     return key < 0 && bconv_targets(j) > 16 ? -2 : key;
 }
 
-void plan_bconv(Plan &P, const std::vector<BConvJob> &jobs)
+void plan_bconv(const fides_ctx *c, Plan &P, const std::vector<BConvJob> &jobs)
 {
     std::vector<bool> done(jobs.size(), false);
+    const bool small = bconv_small(c, jobs, (int)jobs.size());
     for (size_t j = 0; j < jobs.size(); ++j) {
         if (done[j]) continue;
-        const int key = plan_bconv_key(jobs[j]);
+        const int key = small ? 0 : plan_bconv_key(jobs[j]);
         std::vector<BConvJob> g;
         int max_dst = 0, ns = 0;
         for (size_t k = j; k < jobs.size(); ++k) {
-            if (done[k] || plan_bconv_key(jobs[k]) != key) continue;
+            if (done[k] || (!small && plan_bconv_key(jobs[k]) != key)) continue;
             done[k] = true;
             g.push_back(jobs[k]);
             max_dst = std::max(max_dst, bconv_targets(jobs[k]));
@@ -111,6 +112,7 @@ void plan_bconv(Plan &P, const std::vector<BConvJob> &jobs)
         l.kind = L_BCONV;
         l.bc.njob = (int)g.size();
         l.bc.tc = key < 0;
+        if (small) bconv_sources(g, (int)g.size(), &l.bc.ragged);
         if (l.bc.tc)
             for (const BConvJob &x : g) l.bc.tc_smem = std::max(l.bc.tc_smem, bconv_tc_smem(x));
         l.ns = ns;
@@ -274,14 +276,14 @@ void plan_stage(const fides_ctx *c, fides_op *ops, int n_ops, int stage, u64 *co
     }
     plan_tensor(P, tens);
     plan_ntt(P, L_INTT, intt, N, prime_major);
-    plan_bconv(P, up);
+    plan_bconv(c, P, up);
     plan_ntt(P, L_NTT, ntt, N, prime_major);
     plan_inner(P, ip, ip_rows, L_INNER);
     plan_ntt(P, L_INTT, pinv, N, prime_major);
     plan_ntt(P, L_FWD_COLS, fcols, N, prime_major);
     plan_inner(P, ri, ri_rows, L_ROWS_INNER);
     plan_ntt(P, L_INV_COLS, pcols, N, prime_major);
-    plan_bconv(P, down);
+    plan_bconv(c, P, down);
     plan_ntt(P, L_NTT_SUBMUL, fin, N, prime_major);
     plan_ntt(P, L_NTT_SWITCH_SUBMUL, rsfin, N, prime_major);
 }
