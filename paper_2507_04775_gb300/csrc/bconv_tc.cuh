@@ -550,9 +550,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_bconv_tc(BConvArgs A, const P
                                                             const TwPair *__restrict__ c32, int logN, TcPipe pp,
                                                             int *status)
 {
-    // the dependents may launch now; the body waits for the previous kernel
-    // after staging the job's constants
-    pdl_trigger();
+    // (the body waits for the previous kernel after staging the job's constants)
     if (A.djob) bconv_tc_body<FORM>(A.djob[blockIdx.y], P, c32, logN, pp, status);
     else bconv_tc_body<FORM>(A.job[blockIdx.y], P, c32, logN, pp, status);
 }

@@ -65,7 +65,7 @@ __device__ __forceinline__ void store2(u64 *p, u64 x0, u64 x1)
 template <int OP, bool VEC>
 __global__ void __launch_bounds__(256) k_elem(ElemArgs A, const PrimeInfo *__restrict__ P)
 {
-    pdl_enter();
+    pdl_wait();
     const size_t S = (size_t)A.nl << A.logN;     // words of one polynomial
     const bool two_b = OP == E_HADD || OP == E_HSUB;
     const bool pt_b = OP == E_PTADD || OP == E_PTMULT;
@@ -275,7 +275,7 @@ __device__ __forceinline__ void mac_terms(int nt, const PrimeInfo &p, u64 (&s)[W
 template <bool VEC>
 __global__ void __launch_bounds__(256, 3) k_ptmac(MacArgs A, const PrimeInfo *__restrict__ P)
 {
-    pdl_enter();
+    pdl_wait();
     const size_t S = (size_t)A.nl << A.logN;
     // two consecutive words at the same position of both polynomials per
     // step: each plaintext word is read once
@@ -352,7 +352,7 @@ struct CmacArgs {
 template <bool VEC>
 __global__ void __launch_bounds__(256, 4) k_cmac(const CmacArgs A, const PrimeInfo *__restrict__ P)
 {
-    pdl_enter();
+    pdl_wait();
     const size_t S = (size_t)A.nl << A.logN;
     // two words per thread and step (both in one limb: N is even)
     for (size_t v = (size_t)blockIdx.x * blockDim.x + threadIdx.x; v < S; v += (size_t)gridDim.x * blockDim.x) {

@@ -418,23 +418,21 @@ void fides_trace_end(int id, cudaStream_t st);
 void fides_count_launch();
 int fides_trace_set(int on);
 
-// Programmatic dependent launch: every kernel of the library lets the next
-// kernel in its stream launch as soon as all of its CTAs are running, and waits
-// for the previous kernel to finish (and its memory to be visible) before it
-// reads anything a kernel produced.  The next kernel's CTAs thus occupy SMs
-// freed during this kernel's last wave instead of after a launch gap.
-__device__ __forceinline__ void pdl_enter()
+// Programmatic dependent launch: a kernel starts while the one before it still
+// runs, reads what no kernel writes (twiddles, conversion matrices, keys, launch
+// tables uploaded by the host), and waits for its predecessor to finish, and its
+// memory to be visible, before it reads anything a kernel produced.  Only then
+// does it let the next kernel start: one kernel waits at a time.  (Triggering at
+// entry, before the wait, let several successors queue up on the SMs, and single-
+// wave kernels ran up to twice as long between them: a transform of 7 limbs at
+// logN = 16 14.0 us against 7.7, HRotate at logN = 14 58.6 against 43.8.
+// Triggering later, before a kernel's stores, costs large launches the overlap
+// of their last wave: HMult at 30 limbs 238 against 268 us.)
+__device__ __forceinline__ void pdl_wait()
 {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
-
-// The two halves of pdl_enter, for kernels that first read data no kernel
-// writes (twiddles, conversion matrices, keys, launch tables uploaded by the
-// host) so that those reads overlap the previous kernel's last wave: trigger
-// at entry, wait before the first read of anything a kernel produces.
-__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 template <typename... Params, typename... Args>
 inline cudaError_t fides_launch_kernel(void (*kern)(Params...), dim3 grid, dim3 block, cudaStream_t st,

@@ -159,7 +159,6 @@ __device__ __forceinline__ void bconv_body(const BConvJob &B, const PrimeInfo *_
 template <int NS, bool RAG>
 __global__ void __launch_bounds__(256) k_bconv(BConvArgs A, const PrimeInfo *__restrict__ P, int logN, int tg)
 {
-    pdl_trigger();   // the body waits after staging the job's constants
     if (A.djob) bconv_body<NS, RAG>(A.djob[blockIdx.y], P, logN, tg);
     else bconv_body<NS, RAG>(A.job[blockIdx.y], P, logN, tg);
 }
@@ -241,15 +240,16 @@ inline int bconv_targets(const BConvJob &j)
 // one launch whatever their source counts.  The tensor-core kernel's set-up
 // (barriers, tensor memory, the matrix image, four roles to fill) takes longer
 // than few products, and its time per tile hardly depends on the targets, while
-// the integer kernel's grows with them: up to ten targets and 2^22 products in
-// all, or six and 2^24, of at most twelve sources (at logN = 12, where the
-// tensor-core kernel has one tile per CTA, up to four targets).  HMult by integer
-// against tensor-core conversions, us: logN = 16, 10 special primes, 1 limb 57.9
-// 78.7, 4 limbs 71.0 83.3, 6: 85.6 89.6, 8 (10.5 M products in ModDown) 92.3
-// 92.0; logN = 17, 4 + 9 limbs 111.3 121.6; logN = 15, 7 + 7 limbs 53.8 66.1,
-// 14 + 7 (14 targets, 6.4 M) 88.3 82.3; logN = 14, 10 + 10 limbs 52.7 59.1, 7 + 3
-// 51.2 56.5; logN = 13, 12 + 5 limbs (15 targets, 1.2 M) 52.4 51.6; logN = 12,
-// 4 + 4 limbs 34.4 41.6, 6 + 4 (8 targets) 45.0 40.3.
+// the integer kernel's grows with them: up to 16 targets and 2^21 products in
+// all, ten and 2^22, or six and 2^24, of at most twelve sources (at logN = 12,
+// where the tensor-core kernel has one tile per CTA, up to eight targets).
+// HMult by integer against tensor-core conversions, us: logN = 16, 10 special
+// primes, 1 limb 57.6 71.5, 4 limbs 75.8 84.0, 6: 86.9 90.8, 8 (10.5 M products in
+// ModDown) 98.4 93.6; logN = 17, 4 + 9 limbs 113.6 123.8; logN = 15, 7 + 7 limbs
+// 59.9 65.4, 14 + 7 (14 targets, 6.4 M) 85.1 82.2; logN = 14, 7 + 3 limbs 42.2
+// 50.9, 10 + 10 48.2 53.7, 15 + 10 (20 targets, 4.1 M) 68.6 65.2; logN = 13, 14 + 5
+// limbs (15 targets, 1.6 M) 41.2 46.9; logN = 12, 6 + 4 limbs (8 targets) 35.6
+// 39.4, 12 + 4 (12 targets) 43.1 40.5.
 template <class V>
 inline bool bconv_small(const fides_ctx *c, const V &jobs, int n)
 {
@@ -260,7 +260,7 @@ inline bool bconv_small(const fides_ctx *c, const V &jobs, int n)
         work += (long)jobs[j].n_src * bconv_targets(jobs[j]);
         nd = std::max(nd, bconv_targets(jobs[j]));
     }
-    return nd <= (c->logN == 12 ? 4 : 10) && (work << c->logN) <= (nd <= 6 ? 1L << 24 : 1L << 22);
+    return nd <= (c->logN == 12 ? 8 : 16) && (work << c->logN) <= 1L << (nd <= 6 ? 24 : (nd <= 10 ? 22 : 21));
 }
 
 // One integer launch for the jobs, of at most twelve sources each: the largest
@@ -450,7 +450,6 @@ template <int MAXB, bool V2>
 __global__ void __launch_bounds__(256, (MAXB <= 3 ? 4 : 1))
     k_inner(IPArgs A, int L, int nfull, const PrimeInfo *__restrict__ P, int logN)
 {
-    pdl_trigger();   // inner_body waits after issuing its key loads
     const int z = blockIdx.y;
     if (A.dop) {
         const int r = __ldg(A.drow + z);
@@ -496,7 +495,6 @@ template <int MAXB>
 __global__ void __launch_bounds__(256, (MAXB <= 3 ? 4 : 1))
     k_inner_hoist(const __grid_constant__ IPHoistArgs A, int L, int nfull, const PrimeInfo *__restrict__ P, int logN)
 {
-    pdl_trigger();   // inner_body waits after issuing its key loads
     inner_body<MAXB, false>(A.op[blockIdx.y % A.nop], blockIdx.y / A.nop, L, nfull, P, logN);
 }
 
@@ -559,7 +557,7 @@ __device__ __forceinline__ void tensor_body(const TensorOp &o, int limb, const P
 
 __global__ void __launch_bounds__(256) k_tensor(TensorArgs A, const PrimeInfo *__restrict__ P, int logN)
 {
-    pdl_enter();
+    pdl_wait();
     const int z = blockIdx.y;
     if (A.dop) {
         const int k = find_op(A.dpre, A.nop, z);

@@ -43,7 +43,7 @@ __global__ void __launch_bounds__(256) k_hr_last(const u64 *lastc, const u64 *co
                                                  const TwPair *__restrict__ md_pinv, const PrimeInfo *__restrict__ P,
                                                  int l, int N)
 {
-    pdl_enter();
+    pdl_wait();
     const TwPair pinv = md_pinv[l];
     const PrimeInfo p = P[l];
     const int t = blockIdx.y;

@@ -518,7 +518,6 @@ __global__ void __launch_bounds__(ntt_threads<S, KIND, CT, LE>(), MINB)
     // the job table, the primes and the twiddles are the context's or the
     // host's: read (and the column twiddles staged) before waiting for the
     // previous kernel, whose output is read only below
-    pdl_trigger();
     const int t = threadIdx.x;
     const Job J = get_job(set, blockIdx.y, 1 << LOGN);
     const PrimeInfo pr = P[J.prime];

@@ -97,13 +97,15 @@ inline size_t rows_inner_smem(int max_beta)
 
 // Whether key switches of up to `beta` digits over `limbs` extended limbs in all
 // take the fused kernel: two-pass transforms with folding primes (digits below
-// 2q: the cross products of five sum below 5 x 3 x 2^60 < 2^64), and 11 limbs of
-// logN = 16 or more.  Below, a CTA's chain of digits is longer than the launches
-// it saves: HMult at logN = 15 with 14 + 7 limbs 81.9 -> 84.0 us, with 10 + 10
-// equal, with 20 + 10 100.1 -> 96.3; at logN = 16 with 1 + 10 limbs 82.1 -> 78.7.
+// 2q: the cross products of five sum below 5 x 3 x 2^60 < 2^64), and one digit, or
+// 11 limbs of logN = 16 or more.  Below, a CTA's chain of digits is longer than
+// the launches it saves: HMult at logN = 14 with 7 + 3 limbs, three digits, 42.2
+// -> 46.3 us, at logN = 15 with 14 + 7, two digits, 82.9 -> 85.2, with 7 + 7, one
+// digit, 59.9 -> 53.7, with 20 + 10 97.4 -> 94.9; at logN = 16 with 1 + 10 limbs
+// 60.5 -> 57.6, 17 + 10 145.9 -> 141.5.
 inline bool rows_inner_ok(const fides_ctx *c, int beta, int limbs)
 {
-    return c->fold && c->logN > 12 && beta <= 5 && ((long)limbs << c->logN) >= (11L << 16);
+    return c->fold && c->logN > 12 && beta <= 5 && (beta == 1 || ((long)limbs << c->logN) >= (11L << 16));
 }
 
 // Index maps of a tile: C rows of 2^S elements, padded by a word in sixteen.
@@ -207,7 +209,6 @@ __global__ void __launch_bounds__((C << S) >> RI_LE, MAXB <= 3 ? 6 : 5)
     using T = RiTile<S, C>;
     extern __shared__ u64 rsm[];
     constexpr int TILE = C * T::RP;
-    pdl_trigger();
     const int N = 1 << LOGN, nfull = L + K;
     IPOp op;
     int z;

@@ -1,5 +1,5 @@
 """GPU parity of key switches whose conversions go to the integer kernel because
-they are small, on both sides of the rule (ten or six targets, four at logN =
+they are small, on both sides of the rule (16, ten or six targets, eight at logN =
 12) and with ragged last digits, whose jobs share a launch of the largest source
 count: single operations, a batch and round-to-nearest."""
 import numpy as np
@@ -15,8 +15,8 @@ from paper_2507_04775_gb300 import OP_HMULT, Batch, Context, Op, find_primes, to
 
 
 @pytest.mark.parametrize("logN,L,K,dnum,levels", [
-    (12, 6, 2, 3, (1, 3, 4, 5)), (13, 12, 5, 3, (4, 6, 10, 11)), (14, 7, 3, 3, (3, 4, 7)),
-    (13, 12, 12, 1, (12, 7)), (13, 26, 13, 2, (13, 2))])
+    (12, 10, 4, 3, (1, 4, 5, 8, 9, 10)), (13, 14, 5, 3, (4, 6, 11, 14)), (14, 7, 3, 3, (3, 4, 7)),
+    (13, 12, 12, 1, (12, 7)), (13, 26, 13, 2, (13, 2)), (13, 20, 4, 5, (16, 17))])
 @pytest.mark.parametrize("nearest", [False, True])
 def test_small_conversions(logN, L, K, dnum, levels, nearest):
     q = find_primes(logN, 54, L)
