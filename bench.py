@@ -192,12 +192,14 @@ def workload_inputs(P, q, p, seed):
     return A, B, keys
 
 
-def launch_model(nl, K, alpha, N, bconv="k_bconv_tc"):
+def launch_model(nl, K, alpha, N, bconv="k_bconv_tc", rows_inner=False):
     """Per-step launches of the library's kernels with their algorithmic work.
 
     Unit of an NTT pass: one limb (N u64 read + N written = 16 N bytes,
-    (N/2)*log2(N)/2 butterflies = one Shoup product each).  Element-wise
-    kernels count the limbs they must read and write once.  Returns a list of
+    (N/2)*log2(N)/2 butterflies = one product each).  Element-wise
+    kernels count the limbs they must read and write once.  rows_inner: the
+    forward row pass, the inner product and the inverse row pass of the special
+    limbs as one kernel, as large key switches run.  Returns a list of
     (kernel, bytes, modmuls)."""
     W = 8 * N
     half_bfly = (N // 2) * 8          # butterflies of one pass (8 of the 16 stages) per limb
@@ -224,9 +226,14 @@ def launch_model(nl, K, alpha, N, bconv="k_bconv_tc"):
         ntt("inv", nl, ninv=True, first_bytes=fb, first_mm=fm)
         ntgt = beta * ne - nl
         L.append((bconv, W * (nl + ntgt), N * sum(min(alpha, nl - j * alpha) * (ne - min(alpha, nl - j * alpha)) for j in range(beta))))
-        ntt("fwd", ntgt)
-        L.append(("k_inner", W * (beta * ne + 2 * beta * ne + 2 * ne), N * 2 * beta * ne))
-        ntt("inv", 2 * K, ninv=True)                                 # ModDown: P-limbs to coefficients
+        if rows_inner:
+            L.append(("k_ntt_fwd_cols", 2 * W * ntgt, half_bfly * ntgt))
+            L.append(("k_rows_inner", W * (3 * beta * ne + 2 * ne), half_bfly * (ntgt + 2 * K) + N * 2 * beta * ne))
+            L.append(("k_ntt_inv_cols", 2 * W * 2 * K, (half_bfly + N) * 2 * K))
+        else:
+            ntt("fwd", ntgt)
+            L.append(("k_inner", W * (beta * ne + 2 * beta * ne + 2 * ne), N * 2 * beta * ne))
+            ntt("inv", 2 * K, ninv=True)                             # ModDown: P-limbs to coefficients
         L.append((bconv, W * (2 * K + 2 * nl), N * 2 * K * nl))
         extra = W * nl * (2 + mode0 + mode1)                         # aux reads (+ out reads when accumulating)
         ntt("fwd", 2 * nl, extra_bytes=extra, extra_mm=2 * N * nl)
@@ -289,21 +296,20 @@ def peaks():
         return 6800.0, "fallback", 2070.0
 
 
-# ALU roofline of a 64-bit Shoup product, from unit counts and the SM clock:
-# 152 SMs x 64 lanes of the integer multiply (fmaheavy) pipe per clock, and 16
-# lane-cycles per product -- its 10 IMAD-class instructions (4 for the high
-# half of a 64x64 product, 3 for each low half) hold a sub-partition's pipe 32
-# cycles per warp of 32 products (ncu on the register-resident microbenchmark:
-# 10.0 FMA-pipe warp instructions and 1.00 pipe cycle per product per
-# sub-partition, the pipe 95.6 % busy).
-LANE_CYCLES_PER_MODMUL = 16
+# ALU roofline of a modular product, from unit counts and the SM clock: 152 SMs
+# x 64 lanes of the integer multiply (fmaheavy) pipe per clock.  The workload's
+# primes fold (2^k - d just below a power of two): a product is five 32 x 32 -> 64
+# multiplies, which hold a sub-partition's pipe 4 cycles each per warp of 32
+# products, so 10 lane-cycles.  (A Shoup product, which the in-run
+# microbenchmark times, is 10 IMAD-class instructions and 16 lane-cycles.)
+LANE_CYCLES_PER_MODMUL = 10
 FMAHEAVY_LANES_PER_CLK_SM = 64
 SMS = 152
 
 # What limits each kernel, from its ncu profile: the NTT passes the integer
 # multiply pipe, the inner and tensor products DRAM, the conversion the
 # tensor-core issue path.
-KERNEL_BOUND = {"k_ntt": "alu", "k_inner": "hbm", "k_tensor": "hbm", "k_elem": "hbm", "k_ptmac": "hbm",
+KERNEL_BOUND = {"k_ntt": "alu", "k_rows_inner": "alu", "k_inner": "hbm", "k_tensor": "hbm", "k_elem": "hbm", "k_ptmac": "hbm",
                 "k_bconv_tc": "tensor"}
 
 
@@ -464,7 +470,8 @@ def run_fides(args, world, rank, local):
     # ---------------- roofline of the dominant kernel ----------------
     kern = {k: v for k, v in trace.items() if k.startswith("k_")}
     top = max(kern, key=lambda k: kern[k][1])
-    model = launch_model(nl, P.nk, ctx.alpha, N, "k_bconv_tc" if ctx.tensor_bconv else "k_bconv")
+    model = launch_model(nl, P.nk, ctx.alpha, N, "k_bconv_tc" if ctx.tensor_bconv else "k_bconv",
+                         rows_inner="k_rows_inner" in kern)
     per_kernel = {}
     for name, by, mm in model:
         d = per_kernel.setdefault(name, [0, 0, 0])
@@ -473,7 +480,7 @@ def run_fides(args, world, rank, local):
         d[2] += mm
     mismatch = {k: (per_kernel.get(k, [0])[0] * args.steps, kern[k][0]) for k in kern
                 if per_kernel.get(k, [0])[0] * args.steps != kern[k][0]}
-    n_launch, by_step, mm_step = per_kernel[top]
+    n_launch, by_step, mm_step = per_kernel.get(top, (1, 0, 0))
     avg_ms = kern[top][1] / kern[top][0]
     bytes_per_launch = by_step / n_launch
     mm_per_launch = mm_step / n_launch
@@ -488,8 +495,8 @@ def run_fides(args, world, rank, local):
            "frac": round(hbm_ach / hbm_peak, 4), "traffic": traffic, "peak_source": hbm_src}
     alu = {"bound": "alu", "achieved": round(alu_ach, 1), "peak": round(alu_peak, 1), "unit": "Gmodmul/s",
            "frac": round(alu_ach / alu_peak, 4),
-           "peak_source": ("derived: 152 SMs x 64 fmaheavy lanes x %.0f MHz / 16 lane-cycles per Shoup product "
-                           "(10 IMAD-class instructions, 32 pipe cycles per warp; ncu on the microbenchmark)" % sm_max),
+           "peak_source": ("derived: 152 SMs x 64 fmaheavy lanes x %.0f MHz / 10 lane-cycles per folding product "
+                           "(five 32x32->64 multiplies, 20 pipe cycles per warp)" % sm_max),
            "measured_microbenchmark": {
                "peak": round(peak_mm, 1), "frac": round(alu_ach / peak_mm, 4),
                "source": "measured in-run: register-resident Shoup products on all SMs (fides_measure_modmul_peak)"}}
@@ -576,11 +583,11 @@ def run_fides(args, world, rank, local):
         "op_roofline_note": ("compulsory bytes = input ciphertexts + the key limbs in use + outputs, against the "
                              "measured HBM peak; modmul-equivalents = (beta+2)(nl+K) transforms x (N/2) log2 N "
                              "butterflies + conversion multiply-adds + element-wise products, against the derived "
-                             "Shoup-product peak (conversions run on the tensor cores, so alu_frac overstates the "
+                             "folding-product peak (conversions run on the tensor cores, so alu_frac overstates the "
                              "integer pipes' share)"),
         "kernel_roofline_note": ("algorithmic bytes (launch model) / live launch time against the measured HBM peak; "
-                                 "modular products (Shoup butterflies, inner-product and tensor-product multiply-adds) "
-                                 "/ live launch time against the derived Shoup-product peak; k_bconv_tc: fp16 "
+                                 "modular products (butterflies, inner-product and tensor-product multiply-adds) "
+                                 "/ live launch time against the derived folding-product peak; k_bconv_tc: fp16 "
                                  "flops of the MMA shapes it issues against the measured dense bf16 peak (fp16 runs "
                                  "at the bf16 rate); bound: what the kernel's ncu profile shows limits it"),
         "gpu_launches": int(launches),
@@ -1181,7 +1188,8 @@ def load_traffic(kernel, bytes_per_launch):
 KERNEL_SOURCES = {"k_ntt": ["ntt.cuh", "ntt_impl.cuh", "ntt_l16.cu", "fides_internal.cuh"],
                   "k_bconv_tc": ["bconv_tc.cuh", "kernels.cuh", "fides_internal.cuh"],
                   "k_bconv": ["kernels.cuh", "fides_internal.cuh"],
-                  "k_inner": ["kernels.cuh", "fides_internal.cuh"]}
+                  "k_rows_inner": ["rows_inner.cuh", "ntt.cuh", "ntt_impl.cuh", "ntt_l16.cu", "fides_internal.cuh"],
+                  "k_inner": ["kernels.cuh", "rows_inner.cuh", "fides_internal.cuh"]}
 
 
 def sources_sha(kernel: str = "k_ntt") -> str:
