@@ -130,7 +130,7 @@ int fides_find_primes(int logN, int bits, int count, const uint64_t *exclude, in
  *   primes : host array of L q-primes then K special primes, each prime,
  *            = 1 mod 2N, < 2^61, all distinct.
  *   K      : number of special primes, 1 <= K, L + K <= 64.
- * Owns device tables (twiddles with Shoup companions, base-conversion
+ * Owns device tables (twiddles with their companions, base-conversion
  * matrices) and a scratch pool sized for one operation at the top level.
  */
 int fides_ctx_create(int logN, int L, int dnum, const uint64_t *primes, int K, fides_ctx **out);
