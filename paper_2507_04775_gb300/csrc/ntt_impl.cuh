@@ -94,6 +94,23 @@ void launch_pass_v(int v, const fides_ctx *c, const LimbSet &set, const TwPair *
     }
 }
 
+// Variant of a forward row pass.  An epilogue that reads operands (ModDown,
+// Rescale: two or three words a coefficient against one) waits for HBM where
+// the plain pass waits for the multiply pipe.  Past one wave of the
+// 80-register tiles (28 limbs of logN = 16) more warps are worth more than
+// registers, so the same tiles run within 64: HMult by the rows of its ModDown,
+// 80 against 64 registers (folding arithmetic, us), logN = 16, 17 limbs 143.5
+// 140.9, 21: 191.1 189.4, 30: 234.5 231.4; logN = 17, 36 limbs 628.9 622.3.
+// Within that wave they only lose (10 limbs 99.9 105.7), and plain passes of
+// 60 limbs do too (35.1 35.8).
+template <class Epi>
+int fwd_rows_variant(const fides_ctx *c, const LimbSet &set)
+{
+    const int v = variant_of(c, FWD_ROWS, set.total);
+    if (std::is_same_v<Epi, EpiCanon> || ((long)set.total << c->logN) <= 28L << 16) return v;
+    return v == 1 ? 4 : (v == 2 ? 3 : v);
+}
+
 template <int LOGN, class Pro, class Epi>
 int forward(const fides_ctx *c, const LimbSet &set, Pro pro, Epi epi, cudaStream_t st)
 {
@@ -106,7 +123,7 @@ int forward(const fides_ctx *c, const LimbSet &set, Pro pro, Epi epi, cudaStream
     } else {
         launch_pass_v<LOGN, 0, false, false>(variant_of(c, FWD_COLS, set.total), c, set, c->d_tw, pro, EpiLazy{},
                                              st, "k_ntt_fwd_cols");
-        launch_pass_v<LOGN, 1, false, false>(variant_of(c, FWD_ROWS, set.total), c, set, c->d_tw, ProDst{}, epi, st,
+        launch_pass_v<LOGN, 1, false, false>(fwd_rows_variant<Epi>(c, set), c, set, c->d_tw, ProDst{}, epi, st,
                                              "k_ntt_fwd_rows");
     }
     return fides_check_cuda(cudaGetLastError(), "ntt forward launch");
