@@ -377,8 +377,10 @@ int fides_conjugate(fides_ctx *ctx, const fides_ct *a, const fides_key *ck, fide
  *   rks   : host array [n_rot] of key handles, rks[k] registered with g_k
  *   outs  : host array [n_rot] of output descriptors at a->n_limbs; none may
  *           alias a.  out scales are set to a->scale.
- * 1 <= n_rot <= 64.  Uses the context's scratch (one ModUp + one key
- * switch's accumulators); rotations run one after another on `stream`.
+ * 1 <= n_rot <= 64.  Uses the context's scratch (one ModUp and the
+ * accumulators of up to four rotations, as many as it holds); the rotations
+ * run in groups of that many on `stream`, one at a time and in order if
+ * outputs overlap one another.
  */
 int fides_rotate_hoisted(fides_ctx *ctx, const fides_ct *a, int n_rot, const int64_t *steps,
                          const fides_key *const *rks, fides_ct *outs, void *stream);
