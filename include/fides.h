@@ -163,8 +163,8 @@ int fides_ctx_add_stream(fides_ctx *ctx, void *stream);
  * with a 64- or 80-register budget, 16 or 8 elements per thread) of each
  * two-pass transform's pass for every limb count 1..max_limbs (at most 128; larger
  * launches use the choice for 128) on this context's scratch, and keeps the
- * fastest.  Without it the variant goes by the launch's size.  Results are unchanged
- * by the choice.  Synchronises `stream`; do not run it while other work uses
+ * fastest.  Without it the variant goes by the launch's size, whatever its limb
+ * count.  Results are unchanged by the choice.  Synchronises `stream`; do not run it while other work uses
  * this context.  logN = 12 has a single variant (returns FIDES_OK at once).
  * fides_ctx_ntt_tile reports the variant chosen for pass 0..3 (forward
  * columns, forward rows, inverse rows, inverse columns) at n_limbs as
@@ -177,7 +177,8 @@ int fides_ctx_ntt_tile(const fides_ctx *ctx, int pass, int n_limbs);
  * The tuned table itself, for an autotuner cache: FIDES_TUNE_ENTRIES bytes,
  * the variant index per pass kind (4) and limb count (0..128).  set = 0
  * copies the context's table out; set = 1 installs `table` (FIDES_ERR_ARG,
- * nothing changed, if an entry is not a variant index).
+ * nothing changed, if an entry is not a variant index).  Installing the table
+ * that an untuned context gives out restores the choice by size.
  */
 #define FIDES_TUNE_ENTRIES (4 * 129)
 int fides_ctx_tune_table(fides_ctx *ctx, unsigned char *table, int set);

@@ -181,8 +181,10 @@ struct fides_ctx {
     int fold;
 
     // NTT tile variant per pass kind (forward columns, forward rows, inverse
-    // rows, inverse columns) and limb count (ntt.cu)
+    // rows, inverse columns) and limb count (ntt.cu), and whether it was tuned
+    // or installed (otherwise launches go by ntt_default_variant)
     int sms;
+    int ntt_tuned;
     unsigned char ntt_var[4][FIDES_TUNE_MAX + 1];
 };
 

@@ -58,34 +58,19 @@ void tune_one(const fides_ctx *c, int kind, int v, const LimbSet &s, cudaStream_
 }
 }  // namespace
 
-// Default variants before autotuning.  A small launch runs in one wave, whose
-// length is one thread's instruction stream: eight elements per thread halve
-// it and put twice the warps in flight.  Larger launches are bound by the
-// multiply pipe and the twiddle reads, and sixteen elements exchange through
-// shared memory once instead of twice.  The column pass crosses over at 22
-// limbs of logN = 16 (1.4 M elements), the forward row pass, whose twiddles
-// come from L2, at 56, and the inverse row pass not within 120.  Chains of
-// whole transforms, columns + rows with sixteen and sixteen elements per
-// thread, eight and eight, sixteen and eight (folding arithmetic, us):
-//   logN = 16 forward  1 limb 6.5 5.0 5.6, 10: 17.5 14.8 12.8, 20: 20.1 15.9
-//     16.6, 24: 20.2 18.8 18.7, 30: 21.9 22.1 20.9, 60: 37.1 40.2 37.2,
-//     90: 53.0 59.1 53.8
-//   logN = 16 inverse  1: 7.3 5.0 6.2, 20: 22.5 17.6 17.6, 30: 25.8 23.7 23.4,
-//     60: 44.4 43.1 41.1, 90: 63.0 62.3 59.2
-//   logN = 17 forward  7: 15.6 15.4 17.7, 12: 21.3 21.1 20.1, 30: 43.6 44.7 43.7
-//   logN = 14 forward  60: 18.7 14.6 15.4, 90: 19.1 17.1 17.0, 120: 20.5 21.4 19.3
-// Forward columns of more than 128 limbs of logN = 16 run best within 64
-// registers (logN = 17, 90 limbs: 123.7 -> 121.7 us; logN = 16, 120 limbs: 71.2
-// -> 72.2).
+// The table that tells what runs before autotuning (ntt_rules.h; launches of
+// more limbs than it holds go by their size, too).
+void ntt_default_table(const fides_ctx *c, unsigned char (&table)[4][FIDES_TUNE_MAX + 1])
+{
+    for (int kind = 0; kind < 4; ++kind)
+        for (int n = 0; n <= FIDES_TUNE_MAX; ++n)
+            table[kind][n] = (unsigned char)ntt_default_variant(kind, c->logN, n);
+}
+
 void ntt_default_variants(fides_ctx *c)
 {
-    for (int n = 0; n <= FIDES_TUNE_MAX; ++n) {
-        const long elements = (long)n << c->logN;
-        c->ntt_var[FWD_COLS][n] = elements <= (22L << 16) ? 5 : (elements <= (128L << 16) ? 1 : 4);
-        c->ntt_var[INV_COLS][n] = elements <= (22L << 16) ? 5 : 1;
-        c->ntt_var[FWD_ROWS][n] = elements <= (56L << 16) ? 5 : 2;
-        c->ntt_var[INV_ROWS][n] = 5;
-    }
+    ntt_default_table(c, c->ntt_var);
+    c->ntt_tuned = 0;
 }
 
 extern "C" int fides_ctx_autotune(fides_ctx *c, int max_limbs, void *stream)
@@ -135,6 +120,7 @@ extern "C" int fides_ctx_autotune(fides_ctx *c, int max_limbs, void *stream)
     // counts above the tuned range keep the widest tile when it won at the top
     for (int kind = 0; kind < 4; ++kind)
         for (int n = maxn + 1; n <= FIDES_TUNE_MAX; ++n) c->ntt_var[kind][n] = c->ntt_var[kind][maxn];
+    c->ntt_tuned = 1;
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     fides_trace_set(was);
@@ -160,5 +146,9 @@ extern "C" int fides_ctx_tune_table(fides_ctx *c, unsigned char *table, int set)
     for (size_t i = 0; i < n; ++i)
         if (table[i] >= NVAR) return fides_set_error(FIDES_ERR_ARG, "fides_ctx_tune_table: variant %d out of range", table[i]);
     memcpy(c->ntt_var, table, n);
+    // (a default table that was read out and is put back means the defaults)
+    unsigned char def[4][FIDES_TUNE_MAX + 1];
+    ntt_default_table(c, def);
+    c->ntt_tuned = memcmp(c->ntt_var, def, n) != 0;
     return FIDES_OK;
 }

@@ -18,23 +18,16 @@
 
 #include "fides_internal.cuh"
 #include "ntt.cuh"
+#include "ntt_rules.h"
 #include "rows_inner.cuh"
 
 namespace {
 
-// Tile variants: columns or rows per CTA, resident CTAs per SM at 256-element
-// passes, log2 of the elements per thread.  With sixteen elements 3/6/12 CTAs
-// leave up to 80 registers a thread and 16/8 up to 64; with eight, 8 CTAs of
-// 128 threads leave 64.
-constexpr int NVAR = 6;
-constexpr int VAR_CT[NVAR] = {16, 8, 4, 4, 8, 4};
-constexpr int VAR_MINB[NVAR] = {3, 6, 12, 16, 8, 8};
-constexpr int VAR_LE[NVAR] = {4, 4, 4, 4, 4, 3};
-
-enum PassKind { FWD_COLS = 0, FWD_ROWS = 1, INV_ROWS = 2, INV_COLS = 3 };
-
+// Variant of a pass of `total` limbs: the installed table's (launches past its
+// end take its last entry), or by the launch's whole size.
 inline int variant_of(const fides_ctx *c, int kind, int total)
 {
+    if (!c->ntt_tuned) return ntt_default_variant(kind, c->logN, total);
     return c->ntt_var[kind][total > FIDES_TUNE_MAX ? FIDES_TUNE_MAX : total];
 }
 

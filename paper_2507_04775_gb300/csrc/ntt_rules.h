@@ -1,0 +1,49 @@
+// Tile variants of the two-pass transforms and the rule that picks one by the
+// size of a launch.  Host code without CUDA, so that it can be compiled and
+// checked by itself.
+#pragma once
+
+// Columns or rows per CTA, resident CTAs per SM at 256-element passes, log2 of
+// the elements per thread.  With sixteen elements 3/6/12 CTAs leave up to 80
+// registers a thread and 16/8 up to 64; with eight, 8 CTAs of 128 threads leave
+// 64.
+constexpr int NVAR = 6;
+constexpr int VAR_CT[NVAR] = {16, 8, 4, 4, 8, 4};
+constexpr int VAR_MINB[NVAR] = {3, 6, 12, 16, 8, 8};
+constexpr int VAR_LE[NVAR] = {4, 4, 4, 4, 4, 3};
+
+enum PassKind { FWD_COLS = 0, FWD_ROWS = 1, INV_ROWS = 2, INV_COLS = 3 };
+
+// Variant of a pass over `total` limbs where no table was installed.  A small
+// launch runs in one wave, whose length is one thread's instruction stream:
+// eight elements per thread halve it and put twice the warps in flight.  Larger launches are bound by the
+// multiply pipe and the twiddle reads, and sixteen elements exchange through
+// shared memory once instead of twice.  The column pass crosses over at 22
+// limbs of logN = 16 (1.4 M elements; the inverse one at 23: 180 limbs of
+// logN = 13 17.1 against 16.9 us, 24 limbs of logN = 16 20.1 against 20.3), the
+// forward row pass, whose twiddles
+// come from L2, at 56, and the inverse row pass not within 120.  Chains of
+// whole transforms, columns + rows with sixteen and sixteen elements per
+// thread, eight and eight, sixteen and eight (folding arithmetic, us):
+//   logN = 16 forward  1 limb 6.5 5.0 5.6, 10: 17.5 14.8 12.8, 20: 20.1 15.9
+//     16.6, 24: 20.2 18.8 18.7, 30: 21.9 22.1 20.9, 60: 37.1 40.2 37.2,
+//     90: 53.0 59.1 53.8
+//   logN = 16 inverse  1: 7.3 5.0 6.2, 20: 22.5 17.6 17.6, 30: 25.8 23.7 23.4,
+//     60: 44.4 43.1 41.1, 90: 63.0 62.3 59.2
+//   logN = 17 forward  7: 15.6 15.4 17.7, 12: 21.3 21.1 20.1, 30: 43.6 44.7 43.7
+//   logN = 14 forward  60: 18.7 14.6 15.4, 90: 19.1 17.1 17.0, 120: 20.5 21.4 19.3
+// Large forward row passes take four rows a CTA, at logN = 13 eight: four rows
+// of 64 elements are half a warp (480 limbs 43.4 us with four, 32.1 with eight,
+// 32.5 with eight elements a thread; logN = 14 60.6 with four, 65.5).
+// Forward columns of more than 64 limbs of logN = 17 run within 64 registers
+// (90 limbs 125.8 -> 123.5 us; not at logN = 16: 180 limbs 106.3 -> 107.3).
+inline int ntt_default_variant(int kind, int logN, long total)
+{
+    const long elements = total << logN;
+    switch (kind) {
+    case FWD_COLS: return elements <= (22L << 16) ? 5 : (logN == 17 && elements > (128L << 16) ? 4 : 1);
+    case INV_COLS: return elements <= (23L << 16) ? 5 : 1;
+    case FWD_ROWS: return elements <= (56L << 16) ? 5 : (logN == 13 ? 1 : 2);
+    default: return 5;
+    }
+}
