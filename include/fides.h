@@ -163,7 +163,8 @@ int fides_ctx_add_stream(fides_ctx *ctx, void *stream);
  * with a 64- or 80-register budget, 16 or 8 elements per thread) of each
  * two-pass transform's pass for every limb count 1..max_limbs (at most 128; larger
  * launches use the choice for 128) on this context's scratch, and keeps the
- * fastest.  Without it the variant goes by the launch's size, whatever its limb
+ * fastest; forward rows are timed with a plain epilogue and with one that reads
+ * operands (ModDown, Rescale), together, since one choice serves both.  Without it the variant goes by the launch's size, whatever its limb
  * count.  Results are unchanged by the choice.  Synchronises `stream`; do not run it while other work uses
  * this context.  logN = 12 has a single variant (returns FIDES_OK at once).
  * fides_ctx_ntt_tile reports the variant chosen for pass 0..3 (forward

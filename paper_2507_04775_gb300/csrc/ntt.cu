@@ -77,7 +77,6 @@ extern "C" int fides_ctx_autotune(fides_ctx *c, int max_limbs, void *stream)
 {
     if (!c) return fides_set_error(FIDES_ERR_ARG, "fides_ctx_autotune: ctx is NULL");
     if (c->logN == 12) return FIDES_OK;   // one variant only
-    const int np = c->L + c->K;
     const size_t limbs_avail = c->scratch_words / c->N;
     int maxn = std::min(std::min(max_limbs, FIDES_TUNE_MAX), (int)limbs_avail);
     if (maxn < 1) return fides_set_error(FIDES_ERR_ARG, "fides_ctx_autotune: max_limbs < 1");
@@ -90,14 +89,21 @@ extern "C" int fides_ctx_autotune(fides_ctx *c, int max_limbs, void *stream)
     for (int n = 1; n <= maxn && !rc; ++n) {
         LimbSet S;
         memset(&S, 0, sizeof(S));
-        for (int z0 = 0; z0 < n && S.nseg < FIDES_MAX_SEG; z0 += np) {
+        // limbs under the q-primes, in place, with operands (the forward row pass
+        // that reads them) from limbs of the pool that no other segment transforms,
+        // where it has that many
+        for (int z0 = 0; z0 < n && S.nseg < FIDES_MAX_SEG; z0 += c->L) {
             Seg &g = S.seg[S.nseg++];
+            g.count = std::min(c->L, n - z0);
             u64 *p = c->scratch + (size_t)z0 * c->N;
-            g.src = p; g.dst = p; g.aux = nullptr; g.out = nullptr; g.side = nullptr; g.cst = nullptr; g.g = 0;
-            g.count = std::min(np, n - z0); g.prime0 = 0; g.src_step = 1; g.mode = 0; g.pstride = 0;
+            g.aux = c->scratch + std::min((size_t)(n + z0), limbs_avail - g.count) * c->N;
+            g.src = p; g.dst = p; g.out = p; g.side = nullptr; g.cst = nullptr; g.g = 0;
+            g.prime0 = 0; g.src_step = 1; g.mode = 0; g.pstride = 0;
             S.total += g.count;
         }
         for (int kind = 0; kind < 4 && !rc; ++kind) {
+            // (an inverse pass would take the constants for its final scale)
+            for (int i = 0; i < S.nseg; ++i) S.seg[i].cst = kind == FWD_ROWS ? c->d_md_pinv : nullptr;
             float best_ms = 0.f;
             int best = 0;
             for (int v = 0; v < NVAR && !rc; ++v) {

@@ -23,12 +23,11 @@
 
 namespace {
 
-// Variant of a pass of `total` limbs: the installed table's (launches past its
-// end take its last entry), or by the launch's whole size.
-inline int variant_of(const fides_ctx *c, int kind, int total)
+// Variant of a pass of `total` limbs; operands: a forward row pass whose epilogue
+// reads operands.
+inline int variant_of(const fides_ctx *c, int kind, int total, bool operands = false)
 {
-    if (!c->ntt_tuned) return ntt_default_variant(kind, c->logN, total);
-    return c->ntt_var[kind][total > FIDES_TUNE_MAX ? FIDES_TUNE_MAX : total];
+    return ntt_variant(c->ntt_var[kind], FIDES_TUNE_MAX + 1, c->ntt_tuned, kind, c->logN, total, operands);
 }
 
 template <int LOGN>
@@ -87,23 +86,6 @@ void launch_pass_v(int v, const fides_ctx *c, const LimbSet &set, const TwPair *
     }
 }
 
-// Variant of a forward row pass.  An epilogue that reads operands (ModDown,
-// Rescale: two or three words a coefficient against one) waits for HBM where
-// the plain pass waits for the multiply pipe.  Past one wave of the
-// 80-register tiles (28 limbs of logN = 16) more warps are worth more than
-// registers, so the same tiles run within 64: HMult by the rows of its ModDown,
-// 80 against 64 registers (folding arithmetic, us), logN = 16, 17 limbs 143.5
-// 140.9, 21: 191.1 189.4, 30: 234.5 231.4; logN = 17, 36 limbs 628.9 622.3.
-// Within that wave they only lose (10 limbs 99.9 105.7), and plain passes of
-// 60 limbs do too (35.1 35.8).
-template <class Epi>
-int fwd_rows_variant(const fides_ctx *c, const LimbSet &set)
-{
-    const int v = variant_of(c, FWD_ROWS, set.total);
-    if (std::is_same_v<Epi, EpiCanon> || ((long)set.total << c->logN) <= 28L << 16) return v;
-    return v == 1 ? 4 : (v == 2 ? 3 : v);
-}
-
 template <int LOGN, class Pro, class Epi>
 int forward(const fides_ctx *c, const LimbSet &set, Pro pro, Epi epi, cudaStream_t st)
 {
@@ -116,8 +98,9 @@ int forward(const fides_ctx *c, const LimbSet &set, Pro pro, Epi epi, cudaStream
     } else {
         launch_pass_v<LOGN, 0, false, false>(variant_of(c, FWD_COLS, set.total), c, set, c->d_tw, pro, EpiLazy{},
                                              st, "k_ntt_fwd_cols");
-        launch_pass_v<LOGN, 1, false, false>(fwd_rows_variant<Epi>(c, set), c, set, c->d_tw, ProDst{}, epi, st,
-                                             "k_ntt_fwd_rows");
+        constexpr bool operands = !std::is_same_v<Epi, EpiCanon>;
+        launch_pass_v<LOGN, 1, false, false>(variant_of(c, FWD_ROWS, set.total, operands), c, set, c->d_tw, ProDst{},
+                                             epi, st, "k_ntt_fwd_rows");
     }
     return fides_check_cuda(cudaGetLastError(), "ntt forward launch");
 }
@@ -191,7 +174,9 @@ int rows_inner(const fides_ctx *c, const IPArgs &A, int limbs, int max_beta, cud
     return fides_set_error(FIDES_ERR_UNSUPPORTED, "rows + inner product: logN = 12");   // rows_inner_ok is false
 }
 
-// one pass of kind `kind` with variant v (for the autotuner)
+// One pass of kind `kind` with variant v (for the autotuner).  Forward rows run
+// twice, once with an epilogue that reads operands (the segments carry aux, out
+// and constants): one choice serves both.
 template <int LOGN>
 void launch_one(const fides_ctx *c, int kind, int v, const LimbSet &set, cudaStream_t st)
 {
@@ -201,6 +186,7 @@ void launch_one(const fides_ctx *c, int kind, int v, const LimbSet &set, cudaStr
         break;
     case FWD_ROWS:
         launch_pass_v<LOGN, 1, false, false>(v, c, set, c->d_tw, ProDst{}, EpiCanon{}, st, "k_ntt_tune");
+        launch_pass_v<LOGN, 1, false, false>(v, c, set, c->d_tw, ProDst{}, EpiSubMul{}, st, "k_ntt_tune");
         break;
     case INV_ROWS:
         launch_pass_v<LOGN, 1, true, false>(v, c, set, c->d_itw, ProPlain{}, EpiLazy{}, st, "k_ntt_tune");

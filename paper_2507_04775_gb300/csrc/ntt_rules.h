@@ -37,13 +37,33 @@ enum PassKind { FWD_COLS = 0, FWD_ROWS = 1, INV_ROWS = 2, INV_COLS = 3 };
 // 32.5 with eight elements a thread; logN = 14 60.6 with four, 65.5).
 // Forward columns of more than 64 limbs of logN = 17 run within 64 registers
 // (90 limbs 125.8 -> 123.5 us; not at logN = 16: 180 limbs 106.3 -> 107.3).
-inline int ntt_default_variant(int kind, int logN, long total)
+//
+// operands: a forward row pass whose epilogue reads operands (ModDown,
+// Rescale: two or three words a coefficient against one) waits for HBM where
+// the plain pass waits for the multiply pipe.  More warps are worth more than
+// registers there, so the same tiles run within 64: a Rescale by its rows, 80
+// against 64 registers (folding arithmetic, us), logN = 16, 58 limbs 54.6 53.3,
+// 78: 69.6 68.8, 98: 88.3 84.5; logN = 17, 32: 66.1 63.4, 58: 115.9 109.9, 98:
+// 177.7 170.1.  Plain passes lose: a transform
+// of 60 limbs 35.5 36.1.
+inline int ntt_default_variant(int kind, int logN, long total, bool operands = false)
 {
     const long elements = total << logN;
     switch (kind) {
     case FWD_COLS: return elements <= (22L << 16) ? 5 : (logN == 17 && elements > (128L << 16) ? 4 : 1);
     case INV_COLS: return elements <= (23L << 16) ? 5 : 1;
-    case FWD_ROWS: return elements <= (56L << 16) ? 5 : (logN == 13 ? 1 : 2);
+    case FWD_ROWS:
+        if (elements <= (56L << 16)) return 5;
+        return logN == 13 ? (operands ? 4 : 1) : (operands ? 3 : 2);
     default: return 5;
     }
+}
+
+// Variant of a pass: what the tuned or installed table (n entries for the pass
+// kind, limb counts from zero) says, whatever the epilogue, or the default.
+// Launches past the table's end take its last entry.
+inline int ntt_variant(const unsigned char *table, int n, bool tuned, int kind, int logN, int total, bool operands)
+{
+    if (!tuned) return ntt_default_variant(kind, logN, total, operands);
+    return table[total < n ? total : n - 1];
 }

@@ -13,23 +13,30 @@ MAIN = r"""
 #include "ntt_rules.h"
 int main()
 {
-    int kind, logN;
+    int kind, logN, operands, tuned;
     long total;
-    while (scanf("%d %d %ld", &kind, &logN, &total) == 3) printf("%d\n", ntt_default_variant(kind, logN, total));
+    unsigned char table[129];                        // an installed table: the limb count modulo NVAR
+    for (int i = 0; i < 129; ++i) table[i] = (unsigned char)(i % NVAR);
+    while (scanf("%d %d %ld %d %d", &kind, &logN, &total, &operands, &tuned) == 5)
+        printf("%d\n", ntt_variant(table, 129, tuned, kind, logN, (int)total, operands));
 }
 """
 
 
 @pytest.fixture(scope="module")
-def default_variant(tmp_path_factory):
+def variant(tmp_path_factory):
     d = tmp_path_factory.mktemp("rules")
     (d / "main.cpp").write_text(MAIN)
     subprocess.run(["g++", "-std=c++17", "-I" + CSRC, "-o", str(d / "rules"), str(d / "main.cpp")], check=True)
 
-    def ask(kind, logN, total):
-        out = subprocess.run([str(d / "rules")], input="%d %d %d\n" % (kind, logN, total), capture_output=True,
-                             text=True, check=True)
-        return int(out.stdout)
+    def ask(kind, logN, totals, operands=False, tuned=False):
+        """The variant for one limb count, or for each of several."""
+        many = [totals] if isinstance(totals, int) else list(totals)
+        out = subprocess.run([str(d / "rules")], capture_output=True, text=True, check=True,
+                             input="".join("%d %d %d %d %d\n" % (kind, logN, t, operands, tuned) for t in many))
+        got = [int(x) for x in out.stdout.split()]
+        assert len(got) == len(many)
+        return got[0] if isinstance(totals, int) else got
     return ask
 
 
@@ -39,21 +46,27 @@ def threads(v, S):
 
 
 @pytest.mark.parametrize("logN", [13, 14, 15, 16, 17])
-def test_large_launches_take_large_tiles(default_variant, logN):
+def test_large_launches_take_large_tiles(variant, logN):
     """A rule by elements holds past the 128 limbs that a table has entries for:
     the forward rows leave the one-wave tile, the tile is at least a warp, and
     twice the limbs never go back to the tile of small launches."""
-    n = (1 << 26) >> logN
-    assert n > 128 or logN > 15
-    assert default_variant(FWD_ROWS, logN, n) != 5
-    assert default_variant(FWD_COLS, logN, n) != 5
+    n = (1 << 22) >> logN            # 64 limbs of logN = 16
     S_row = {13: 6, 14: 7, 15: 7, 16: 8, 17: 8}[logN]
-    for kind, S in ((FWD_ROWS, S_row), (INV_ROWS, S_row), (FWD_COLS, logN - S_row), (INV_COLS, logN - S_row)):
-        left = False
-        for total in range(1, 1025):
-            v = default_variant(kind, logN, total) if total % 31 == 1 or total > 1020 else None
-            if v is None:
-                continue
-            assert threads(v, S) >= 32
-            assert not (left and v == 5)
-            left = left or v != 5
+    for kind, S, op in ((FWD_ROWS, S_row, 0), (FWD_ROWS, S_row, 1), (INV_ROWS, S_row, 0), (FWD_COLS, logN - S_row, 0),
+                        (INV_COLS, logN - S_row, 0)):
+        got = variant(kind, logN, range(1, 1025), op)
+        assert min(threads(v, S) for v in got) >= 32
+        if 5 in got and got[-1] != 5:
+            first = next(i for i, v in enumerate(got) if v != 5)
+            assert 5 not in got[first:]
+        assert got[n - 1] != 5 or kind == INV_ROWS
+
+
+@pytest.mark.parametrize("logN", [13, 14, 15, 16, 17])
+def test_an_installed_table_decides_every_pass(variant, logN):
+    """Every entry is what runs, with and without an epilogue that reads
+    operands, and the last one past the table's end."""
+    for kind in range(4):
+        for operands in (False, True):
+            got = variant(kind, logN, range(0, 300), operands, tuned=True)
+            assert got == [min(i, 128) % 6 for i in range(300)]
