@@ -167,9 +167,12 @@ int fides_ctx_add_stream(fides_ctx *ctx, void *stream);
  * operands (ModDown, Rescale), together, since one choice serves both.  Without it the variant goes by the launch's size, whatever its limb
  * count.  Results are unchanged by the choice.  Synchronises `stream`; do not run it while other work uses
  * this context.  logN = 12 has a single variant (returns FIDES_OK at once).
- * fides_ctx_ntt_tile reports the variant chosen for pass 0..3 (forward
- * columns, forward rows, inverse rows, inverse columns) at n_limbs as
- * (tile width << 8) | resident CTAs per SM.
+ * fides_ctx_ntt_tile reports the tile that runs for pass 0..3 (forward
+ * columns, forward rows with a plain epilogue, inverse rows, inverse columns) at
+ * n_limbs as (tile width << 8) | resident CTAs per SM, the latter the target
+ * that the kernel is compiled for.  Contexts with Shoup arithmetic (a prime that
+ * is not 2^k - d with 50 <= k <= 60, d < 2^28) compile fewer tiles, and several
+ * variants run the same one.
  */
 int fides_ctx_autotune(fides_ctx *ctx, int max_limbs, void *stream);
 int fides_ctx_ntt_tile(const fides_ctx *ctx, int pass, int n_limbs);

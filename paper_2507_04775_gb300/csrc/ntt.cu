@@ -136,9 +136,10 @@ extern "C" int fides_ctx_autotune(fides_ctx *c, int max_limbs, void *stream)
 extern "C" int fides_ctx_ntt_tile(const fides_ctx *c, int pass, int n_limbs)
 {
     if (!c || pass < 0 || pass > 3 || n_limbs < 0) return 0;
-    if (c->logN == 12) return (1 << 8) | 3;
-    const int v = variant_of(c, pass, n_limbs);
-    return (VAR_CT[v] << 8) | VAR_MINB[v];
+    if (c->logN == 12) return (1 << 8) | NTT_LIMB_CTAS;
+    const int v = ntt_compiled(variant_of(c, pass, n_limbs), c->fold);
+    const int S = pass == FWD_COLS || pass == INV_COLS ? ntt_col_stages(c->logN) : ntt_row_stages(c->logN);
+    return (ntt_tile_width(v, S) << 8) | ntt_tile_ctas(v, S);
 }
 
 extern "C" int fides_ctx_tune_table(fides_ctx *c, unsigned char *table, int set)

@@ -32,21 +32,8 @@ inline int variant_of(const fides_ctx *c, int kind, int total, bool operands = f
 
 template <int LOGN>
 struct Split {
-    static constexpr int COL = LOGN <= 14 ? 7 : (LOGN <= 16 ? 8 : 9);
-    static constexpr int ROW = LOGN - COL;
-};
-
-// Tile of variant V for a pass of S stages: at most 8 sub-transforms per CTA
-// when they have 512 elements (static shared memory), and the resident-CTA
-// target that keeps the threads per SM (hence the register budget) of the
-// variant's 256-element form.
-template <int V, int S>
-struct Tile {
-    static constexpr int CT = (S >= 9 && VAR_CT[V] > 8) ? 8 : VAR_CT[V];
-    static constexpr int LE = VAR_LE[V];
-    static constexpr int THREADS = (CT << S) >> LE;
-    static constexpr int WANT = (((256 * VAR_CT[V]) >> LE) * VAR_MINB[V]) / THREADS;
-    static constexpr int MINB = WANT < 1 ? 1 : (WANT > 32 ? 32 : WANT);
+    static constexpr int COL = ntt_col_stages(LOGN);
+    static constexpr int ROW = ntt_row_stages(LOGN);
 };
 
 template <int LOGN, int V, int KIND, bool INV, bool NINV, bool FOLD, class Pro, class Epi>
@@ -54,9 +41,9 @@ void launch_pass(const fides_ctx *c, const LimbSet &set, const TwPair *tw, Pro p
                  const char *name)
 {
     constexpr int S = KIND == 0 ? Split<LOGN>::COL : Split<LOGN>::ROW;
-    using T = Tile<V, S>;
-    auto k = k_ntt<LOGN, S, KIND, INV, NINV, T::CT, T::MINB, T::LE, FOLD, Pro, Epi>;
-    dim3 grid((1 << (LOGN - S)) / T::CT, set.total), block(T::THREADS);
+    constexpr int CT = ntt_tile_width(V, S);
+    auto k = k_ntt<LOGN, S, KIND, INV, NINV, CT, ntt_tile_ctas(V, S), VAR_LE[V], FOLD, Pro, Epi>;
+    dim3 grid((1 << (LOGN - S)) / CT, set.total), block(ntt_tile_threads(V, S));
     FIDES_LAUNCH(name, st, k, grid, block, set, (const PrimeInfo *)c->d_prime, tw, pro, epi);
 }
 
@@ -75,13 +62,9 @@ void launch_pass_v(int v, const fides_ctx *c, const LimbSet &set, const TwPair *
         }
         return;
     }
-    // Shoup arithmetic: the wide and the 64-register tiles run as 1 and 2
-    switch (v) {
-    case 0:
-    case 1:
-    case 4: launch_pass<LOGN, 1, KIND, INV, NINV, false>(c, set, tw, pro, epi, st, name); break;
-    case 2:
-    case 3: launch_pass<LOGN, 2, KIND, INV, NINV, false>(c, set, tw, pro, epi, st, name); break;
+    switch (ntt_compiled(v, false)) {
+    case 1: launch_pass<LOGN, 1, KIND, INV, NINV, false>(c, set, tw, pro, epi, st, name); break;
+    case 2: launch_pass<LOGN, 2, KIND, INV, NINV, false>(c, set, tw, pro, epi, st, name); break;
     default: launch_pass<LOGN, 5, KIND, INV, NINV, false>(c, set, tw, pro, epi, st, name); break;
     }
 }
@@ -91,8 +74,8 @@ int forward(const fides_ctx *c, const LimbSet &set, Pro pro, Epi epi, cudaStream
 {
     if (set.total == 0) return FIDES_OK;
     if constexpr (LOGN == 12) {
-        auto k = c->fold ? k_ntt<12, 12, 2, false, false, 16, 2, 3, true, Pro, Epi>
-                         : k_ntt<12, 12, 2, false, false, 16, 2, 3, false, Pro, Epi>;
+        auto k = c->fold ? k_ntt<12, 12, 2, false, false, 16, NTT_LIMB_CTAS, 3, true, Pro, Epi>
+                         : k_ntt<12, 12, 2, false, false, 16, NTT_LIMB_CTAS, 3, false, Pro, Epi>;
         FIDES_LAUNCH("k_ntt_fwd_limb", st, k, dim3(1, set.total), dim3(512), set, (const PrimeInfo *)c->d_prime,
                      (const TwPair *)c->d_tw, pro, epi);
     } else {
@@ -110,8 +93,8 @@ int inverse(const fides_ctx *c, const LimbSet &set, Pro pro, Epi epi, cudaStream
 {
     if (set.total == 0) return FIDES_OK;
     if constexpr (LOGN == 12) {
-        auto k = c->fold ? k_ntt<12, 12, 2, true, true, 16, 2, 3, true, Pro, Epi>
-                         : k_ntt<12, 12, 2, true, true, 16, 2, 3, false, Pro, Epi>;
+        auto k = c->fold ? k_ntt<12, 12, 2, true, true, 16, NTT_LIMB_CTAS, 3, true, Pro, Epi>
+                         : k_ntt<12, 12, 2, true, true, 16, NTT_LIMB_CTAS, 3, false, Pro, Epi>;
         FIDES_LAUNCH("k_ntt_inv_limb", st, k, dim3(1, set.total), dim3(512), set, (const PrimeInfo *)c->d_prime,
                      (const TwPair *)c->d_itw, pro, epi);
     } else {

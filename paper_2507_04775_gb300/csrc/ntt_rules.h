@@ -14,6 +14,32 @@ constexpr int VAR_LE[NVAR] = {4, 4, 4, 4, 4, 3};
 
 enum PassKind { FWD_COLS = 0, FWD_ROWS = 1, INV_ROWS = 2, INV_COLS = 3 };
 
+// Tile of variant v for a pass of S stages: at most 8 sub-transforms per CTA
+// when they have 512 elements (static shared memory), and the resident-CTA
+// target that keeps the threads per SM (hence the register budget) of the
+// variant's 256-element form.
+constexpr int ntt_tile_width(int v, int S) { return S >= 9 && VAR_CT[v] > 8 ? 8 : VAR_CT[v]; }
+constexpr int ntt_tile_threads(int v, int S) { return (ntt_tile_width(v, S) << S) >> VAR_LE[v]; }
+constexpr int ntt_tile_ctas(int v, int S)
+{
+    const int want = (((256 * VAR_CT[v]) >> VAR_LE[v]) * VAR_MINB[v]) / ntt_tile_threads(v, S);
+    return want < 1 ? 1 : (want > 32 ? 32 : want);
+}
+
+// Resident-CTA target of the whole-limb pass of logN = 12 (512 threads).
+constexpr int NTT_LIMB_CTAS = 2;
+
+// Stages of the column and of the row pass.
+constexpr int ntt_col_stages(int logN) { return logN <= 14 ? 7 : (logN <= 16 ? 8 : 9); }
+constexpr int ntt_row_stages(int logN) { return logN - ntt_col_stages(logN); }
+
+// The compiled tile that runs for variant v: with Shoup arithmetic the wide and
+// the 64-register tiles run as 1 and 2.
+constexpr int ntt_compiled(int v, bool fold)
+{
+    return fold ? v : (v == 0 || v == 4 ? 1 : (v == 3 ? 2 : v));
+}
+
 // Variant of a pass over `total` limbs where no table was installed.  A small
 // launch runs in one wave, whose length is one thread's instruction stream:
 // eight elements per thread halve it and put twice the warps in flight.  Larger launches are bound by the

@@ -405,7 +405,8 @@ class Context:
         _check(lib().fides_ctx_tune_table(self._h, ctypes.create_string_buffer(bytes(table), 4 * 129), 1))
 
     def ntt_tile(self, pass_kind: int, n_limbs: int) -> int:
-        """Tile width chosen for pass 0..3 (fwd cols, fwd rows, inv rows, inv cols)."""
+        """Tile that runs for pass 0..3 (fwd cols, fwd rows, inv rows, inv cols):
+        (tile width << 8) | resident CTAs per SM."""
         return int(lib().fides_ctx_ntt_tile(self._h, pass_kind, n_limbs))
 
     # -- primitives --------------------------------------------------------

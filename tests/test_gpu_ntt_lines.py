@@ -48,7 +48,28 @@ def test_reported_tile_past_the_table(logN, limbs):
     assert g.ntt_tile(1, limbs) != small and g.ntt_tile(1, limbs) >> 8 == (8 if logN == 13 else 4)
     table = g.tune_table()
     g.set_tune_table(bytes([2]) * len(table))       # an installed table: its last entry beyond it
-    assert g.ntt_tile(1, limbs) == g.ntt_tile(1, 128) != small
+    assert g.ntt_tile(1, limbs) == g.ntt_tile(1, 128)
     g.set_tune_table(table)                          # the default one put back
     assert g.ntt_tile(1, limbs) != small and g.ntt_tile(1, 60) == small
     g.close()
+
+
+def test_reported_tile_is_the_one_that_runs():
+    """(tile width << 8) | resident CTAs: a context with Shoup arithmetic runs the
+    wide tile as eight columns; 512-element columns (logN = 17) come eight at
+    most, 64-element rows (logN = 13) keep the threads per SM; logN = 12 has one
+    tile, of which two fit."""
+    def tiles(logN, bits, v):
+        q = find_primes(logN, bits, 2)
+        g = Context(logN, q[:1], q[1:], 1)
+        g.set_tune_table(bytes([v]) * len(g.tune_table()))
+        got = [g.ntt_tile(k, 30) for k in range(4)]
+        g.close()
+        return [(t >> 8, t & 255) for t in got]
+
+    assert tiles(16, 54, 0) == [(16, 3)] * 4
+    assert tiles(16, 61, 0) == [(8, 6)] * 4
+    assert tiles(16, 61, 3) == [(4, 12)] * 4
+    assert tiles(17, 54, 0) == [(8, 3), (16, 3), (16, 3), (8, 3)]
+    assert tiles(13, 54, 5) == [(4, 16), (4, 32), (4, 32), (4, 16)]
+    assert tiles(12, 54, 0) == [(1, 2)] * 4
