@@ -137,7 +137,7 @@ extern "C" int fides_ctx_ntt_tile(const fides_ctx *c, int pass, int n_limbs)
 {
     if (!c || pass < 0 || pass > 3 || n_limbs < 0) return 0;
     if (c->logN == 12) return (1 << 8) | NTT_LIMB_CTAS;
-    const int v = ntt_compiled(variant_of(c, pass, n_limbs), c->fold);
+    const int v = ntt_compiled(variant_of(c, pass, n_limbs), c->fold, pass);
     const int S = pass == FWD_COLS || pass == INV_COLS ? ntt_col_stages(c->logN) : ntt_row_stages(c->logN);
     return (ntt_tile_width(v, S) << 8) | ntt_tile_ctas(v, S);
 }

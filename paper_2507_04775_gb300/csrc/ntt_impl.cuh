@@ -62,9 +62,13 @@ void launch_pass_v(int v, const fides_ctx *c, const LimbSet &set, const TwPair *
         }
         return;
     }
-    switch (ntt_compiled(v, false)) {
+    constexpr int kind = KIND == 0 ? (INV ? INV_COLS : FWD_COLS) : (INV ? INV_ROWS : FWD_ROWS);
+    switch (ntt_compiled(v, false, kind)) {
     case 1: launch_pass<LOGN, 1, KIND, INV, NINV, false>(c, set, tw, pro, epi, st, name); break;
     case 2: launch_pass<LOGN, 2, KIND, INV, NINV, false>(c, set, tw, pro, epi, st, name); break;
+    case 4:
+        if constexpr (kind == FWD_COLS) launch_pass<LOGN, 4, KIND, INV, NINV, false>(c, set, tw, pro, epi, st, name);
+        break;
     default: launch_pass<LOGN, 5, KIND, INV, NINV, false>(c, set, tw, pro, epi, st, name); break;
     }
 }

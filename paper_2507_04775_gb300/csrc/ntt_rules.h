@@ -33,11 +33,14 @@ constexpr int NTT_LIMB_CTAS = 2;
 constexpr int ntt_col_stages(int logN) { return logN <= 14 ? 7 : (logN <= 16 ? 8 : 9); }
 constexpr int ntt_row_stages(int logN) { return logN - ntt_col_stages(logN); }
 
-// The compiled tile that runs for variant v: with Shoup arithmetic the wide and
-// the 64-register tiles run as 1 and 2.
-constexpr int ntt_compiled(int v, bool fold)
+// The compiled tile that runs for variant v of a pass: with Shoup arithmetic the
+// wide tile and, but for forward columns, the 64-register ones run as 1 and 2.
+// (Forward transforms at 61-bit primes, columns within 80 against 64 registers,
+// us: logN = 16, 30 limbs 25.9 26.3, 60: 43.8 42.8, 90: 65.3 63.8, 120: 86.2 84.8;
+// logN = 17, 60: 98.2 95.9, 90: 144.6 140.5.)
+constexpr int ntt_compiled(int v, bool fold, int kind)
 {
-    return fold ? v : (v == 0 || v == 4 ? 1 : (v == 3 ? 2 : v));
+    return fold || (v == 4 && kind == FWD_COLS) ? v : (v == 0 || v == 4 ? 1 : (v == 3 ? 2 : v));
 }
 
 // Variant of a pass over `total` limbs where no table was installed.  A small

@@ -70,6 +70,7 @@ def test_reported_tile_is_the_one_that_runs():
     assert tiles(16, 54, 0) == [(16, 3)] * 4
     assert tiles(16, 61, 0) == [(8, 6)] * 4
     assert tiles(16, 61, 3) == [(4, 12)] * 4
+    assert tiles(16, 61, 4) == [(8, 8), (8, 6), (8, 6), (8, 6)]
     assert tiles(17, 54, 0) == [(8, 3), (16, 3), (16, 3), (8, 3)]
     assert tiles(13, 54, 5) == [(4, 16), (4, 32), (4, 32), (4, 16)]
     assert tiles(12, 54, 0) == [(1, 2)] * 4
