@@ -64,7 +64,7 @@ void ntt_default_table(const fides_ctx *c, unsigned char (&table)[4][FIDES_TUNE_
 {
     for (int kind = 0; kind < 4; ++kind)
         for (int n = 0; n <= FIDES_TUNE_MAX; ++n)
-            table[kind][n] = (unsigned char)ntt_default_variant(kind, c->logN, n);
+            table[kind][n] = (unsigned char)ntt_default_variant(kind, c->logN, c->fold, n);
 }
 
 void ntt_default_variants(fides_ctx *c)

@@ -27,7 +27,8 @@ namespace {
 // reads operands.
 inline int variant_of(const fides_ctx *c, int kind, int total, bool operands = false)
 {
-    return ntt_variant(c->ntt_var[kind], FIDES_TUNE_MAX + 1, c->ntt_tuned, kind, c->logN, total, operands);
+    return ntt_variant(c->ntt_var[kind], FIDES_TUNE_MAX + 1, c->ntt_tuned, kind, c->logN, c->fold, total,
+                       operands);
 }
 
 template <int LOGN>

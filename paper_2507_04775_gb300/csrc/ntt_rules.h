@@ -45,54 +45,64 @@ constexpr int ntt_compiled(int v, bool fold, int kind)
 
 // Variant of a pass over `total` limbs where no table was installed.  A small
 // launch runs in one wave, whose length is one thread's instruction stream:
-// eight elements per thread halve it and put twice the warps in flight.  Larger launches are bound by the
-// multiply pipe and the twiddle reads, and sixteen elements exchange through
-// shared memory once instead of twice.  The column pass crosses over at 22
-// limbs of logN = 16 (1.4 M elements; the inverse one at 23: 180 limbs of
-// logN = 13 17.1 against 16.9 us, 24 limbs of logN = 16 20.1 against 20.3), the
-// forward row pass, whose twiddles
-// come from L2, at 56, and the inverse row pass not within 120.  Chains of
-// whole transforms, columns + rows with sixteen and sixteen elements per
-// thread, eight and eight, sixteen and eight (folding arithmetic, us):
-//   logN = 16 forward  1 limb 6.5 5.0 5.6, 10: 17.5 14.8 12.8, 20: 20.1 15.9
-//     16.6, 24: 20.2 18.8 18.7, 30: 21.9 22.1 20.9, 60: 37.1 40.2 37.2,
-//     90: 53.0 59.1 53.8
-//   logN = 16 inverse  1: 7.3 5.0 6.2, 20: 22.5 17.6 17.6, 30: 25.8 23.7 23.4,
-//     60: 44.4 43.1 41.1, 90: 63.0 62.3 59.2
-//   logN = 17 forward  7: 15.6 15.4 17.7, 12: 21.3 21.1 20.1, 30: 43.6 44.7 43.7
-//   logN = 14 forward  60: 18.7 14.6 15.4, 90: 19.1 17.1 17.0, 120: 20.5 21.4 19.3
-// Large forward row passes take four rows a CTA, at logN = 13 eight: four rows
-// of 64 elements are half a warp (480 limbs 43.4 us with four, 32.1 with eight,
-// 32.5 with eight elements a thread; logN = 14 60.6 with four, 65.5).
-// Forward columns of more than 64 limbs of logN = 17 run within 64 registers
-// (90 limbs 125.8 -> 123.5 us; not at logN = 16: 180 limbs 106.3 -> 107.3).
+// eight elements per thread halve it and put twice the warps in flight.  Larger
+// launches are bound by the multiply pipe and the twiddle reads, and sixteen
+// elements exchange through shared memory once instead of twice.  The lines
+// below, in limbs of logN = 16 (as many elements at other degrees), are where
+// chains of whole transforms cross over, eight against sixteen elements in one
+// of the passes (us):
+//   forward columns, 22: folding, logN = 16, 22 limbs 17.6 18.5, 24: 19.1 18.7;
+//     logN = 17, 11: 19.1 19.9, 12: 21.5 20.5; logN = 15, 40: 15.8 15.8, 60: 21.6
+//     20.1.  Shoup, 20: 19.1 19.1, 24: 22.2 21.9
+//   inverse columns, 23: folding, logN = 13, 180: 16.9 17.1; logN = 16, 24: 20.3
+//     20.1; logN = 15, 60: 22.8 22.4.  Shoup, logN = 13, 180: 18.7 19.9; logN = 16,
+//     24: 23.5 23.4
+//   forward rows, 28 folding and 32 Shoup: folding, logN = 16, 24: 18.5 19.3, 30:
+//     21.2 20.7, 36: 24.6 23.2, 60: 37.8 35.5; logN = 14, 90: 17.0 17.9, 120: 19.3
+//     19.1, 240: 34.2 32.2; logN = 17, 12: 20.6 20.5, 20: 31.0 30.1.  Shoup, 30: 25.7
+//     25.9, 36: 29.4 28.3
+//   inverse rows, 32: folding, logN = 16, 24: 20.1 20.2, 30: 23.4 23.2, 36: 26.7
+//     25.7, 60: 41.2 39.4, 120: 82.2 79.6; logN = 15, 60: 22.4 22.8, 90: 30.7 30.4;
+//     logN = 17, 20: 32.9 32.2, 60: 94.4 90.4.  Shoup, 30: 27.5 27.7, 36: 31.4 30.8
+// Large row passes take four rows a CTA, at logN = 13 eight: four rows of 64
+// elements are half a warp (480 limbs forward 43.4 us with four, 32.1 with eight).
+// Forward columns run within 64 registers at logN = 17 past 12 limbs (80 against
+// 64: 12 limbs 20.5 20.7, 15: 25.2 24.7, 30: 43.4 43.2, 60: 85.0 83.9, 90: 125.8
+// 123.5; not at logN = 16: 60 limbs 35.4 35.7, 180: 106.3 107.3), with Shoup
+// products past 44 of logN = 16 (30: 25.9 26.3, 60: 43.8 42.8, 90: 65.3 63.8; logN =
+// 15, 60: 24.3 25.5, 90: 32.9 32.5).
 //
 // operands: a forward row pass whose epilogue reads operands (ModDown,
 // Rescale: two or three words a coefficient against one) waits for HBM where
 // the plain pass waits for the multiply pipe.  More warps are worth more than
-// registers there, so the same tiles run within 64: a Rescale by its rows, 80
-// against 64 registers (folding arithmetic, us), logN = 16, 58 limbs 54.6 53.3,
-// 78: 69.6 68.8, 98: 88.3 84.5; logN = 17, 32: 66.1 63.4, 58: 115.9 109.9, 98:
-// 177.7 170.1.  Plain passes lose: a transform
-// of 60 limbs 35.5 36.1.
-inline int ntt_default_variant(int kind, int logN, long total, bool operands = false)
+// registers there.  With Shoup products the eight-element tile stays ahead at
+// every size measured (a Rescale by its rows, eight and sixteen elements, logN =
+// 16, 58: 62.0 64.6, 98: 98.3 102.4; logN = 17, 98: 196.6 205.9); folding ones
+// cross over at 56 and then run sixteen elements within 64 registers (a Rescale,
+// eight elements, sixteen within 80 and within 64: logN = 16, 46: 44.8 43.9 43.6,
+// 58: 54.4 54.6 53.3, 98: 87.6 88.3 84.5; logN = 17, 32: 64.7 66.1 63.4, 98: 175.9
+// 177.7 170.1; an HRotate, logN = 16, 48: 194.6 196.4 195.9, 56: 210.8 211.4 212.0,
+// 72: 310.0 316.7 308.8).
+inline int ntt_default_variant(int kind, int logN, bool fold, long total, bool operands = false)
 {
-    const long elements = total << logN;
+    const long limbs = ((total << logN) + 65535) >> 16;   // of logN = 16, rounded up
+    const int rows16 = logN == 13 ? 1 : 2;                // row passes with sixteen elements
     switch (kind) {
-    case FWD_COLS: return elements <= (22L << 16) ? 5 : (logN == 17 && elements > (128L << 16) ? 4 : 1);
-    case INV_COLS: return elements <= (23L << 16) ? 5 : 1;
+    case FWD_COLS: return limbs <= 22 ? 5 : (limbs > (logN == 17 ? 24 : 44) && (logN == 17 || !fold) ? 4 : 1);
+    case INV_COLS: return limbs <= 23 ? 5 : 1;
     case FWD_ROWS:
-        if (elements <= (56L << 16)) return 5;
-        return logN == 13 ? (operands ? 4 : 1) : (operands ? 3 : 2);
-    default: return 5;
+        if (operands) return !fold || limbs <= 56 ? 5 : (logN == 13 ? 4 : 3);
+        return limbs <= (fold ? 28 : 32) ? 5 : rows16;
+    default: return limbs <= 32 ? 5 : rows16;
     }
 }
 
 // Variant of a pass: what the tuned or installed table (n entries for the pass
 // kind, limb counts from zero) says, whatever the epilogue, or the default.
 // Launches past the table's end take its last entry.
-inline int ntt_variant(const unsigned char *table, int n, bool tuned, int kind, int logN, int total, bool operands)
+inline int ntt_variant(const unsigned char *table, int n, bool tuned, int kind, int logN, bool fold, int total,
+                       bool operands)
 {
-    if (!tuned) return ntt_default_variant(kind, logN, total, operands);
+    if (!tuned) return ntt_default_variant(kind, logN, fold, total, operands);
     return table[total < n ? total : n - 1];
 }

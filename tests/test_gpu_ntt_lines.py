@@ -12,10 +12,11 @@ pytestmark = pytest.mark.gpu
 from paper_2507_04775_gb300 import Context, find_primes, to_device, to_host  # noqa: E402
 
 
-# limbs of one polynomial, polynomials: on both sides of 22 and 56 limbs of
-# logN = 16, of 128 limbs, and of 64 limbs of logN = 17
-@pytest.mark.parametrize("logN,n,batches", [(16, 11, (2, 6)), (16, 23, (1,)), (16, 19, (3,)), (17, 11, (1,)), (17, 12, (1,)),
-                                            (17, 13, (4, 5)), (14, 16, (8, 14, 15)), (13, 20, (6, 7, 23))])
+# limbs of one polynomial, polynomials: on both sides of 22, 23, 28, 32 and 44
+# limbs of logN = 16 (12 of logN = 17), and of 128 limbs
+@pytest.mark.parametrize("logN,n,batches", [
+    (16, 11, (2, 4, 5)), (16, 23, (1,)), (16, 24, (1,)), (16, 14, (2,)), (16, 29, (1,)), (16, 16, (2,)), (16, 33, (1,)),
+    (17, 11, (1,)), (17, 12, (1,)), (17, 13, (1,)), (14, 16, (8, 14, 15)), (13, 20, (6, 7, 23))])
 @pytest.mark.parametrize("bits", [54, 61])          # folding arithmetic, Shoup products
 def test_both_sides_of_the_lines(logN, n, batches, bits):
     q = find_primes(logN, bits, n)

@@ -13,12 +13,12 @@ MAIN = r"""
 #include "ntt_rules.h"
 int main()
 {
-    int kind, logN, operands, tuned;
+    int kind, logN, fold, operands, tuned;
     long total;
     unsigned char table[129];                        // an installed table: the limb count modulo NVAR
     for (int i = 0; i < 129; ++i) table[i] = (unsigned char)(i % NVAR);
-    while (scanf("%d %d %ld %d %d", &kind, &logN, &total, &operands, &tuned) == 5)
-        printf("%d\n", ntt_variant(table, 129, tuned, kind, logN, (int)total, operands));
+    while (scanf("%d %d %d %ld %d %d", &kind, &logN, &fold, &total, &operands, &tuned) == 6)
+        printf("%d\n", ntt_variant(table, 129, tuned, kind, logN, fold, (int)total, operands));
 }
 """
 
@@ -29,11 +29,12 @@ def variant(tmp_path_factory):
     (d / "main.cpp").write_text(MAIN)
     subprocess.run(["g++", "-std=c++17", "-I" + CSRC, "-o", str(d / "rules"), str(d / "main.cpp")], check=True)
 
-    def ask(kind, logN, totals, operands=False, tuned=False):
+    def ask(kind, logN, totals, operands=False, tuned=False, fold=True):
         """The variant for one limb count, or for each of several."""
         many = [totals] if isinstance(totals, int) else list(totals)
         out = subprocess.run([str(d / "rules")], capture_output=True, text=True, check=True,
-                             input="".join("%d %d %d %d %d\n" % (kind, logN, t, operands, tuned) for t in many))
+                             input="".join("%d %d %d %d %d %d\n" % (kind, logN, fold, t, operands, tuned)
+                                           for t in many))
         got = [int(x) for x in out.stdout.split()]
         assert len(got) == len(many)
         return got[0] if isinstance(totals, int) else got
@@ -59,7 +60,19 @@ def test_large_launches_take_large_tiles(variant, logN):
         if 5 in got and got[-1] != 5:
             first = next(i for i, v in enumerate(got) if v != 5)
             assert 5 not in got[first:]
-        assert got[n - 1] != 5 or kind == INV_ROWS
+        assert got[n - 1] != 5
+
+
+@pytest.mark.parametrize("fold", [True, False])
+def test_lines(variant, fold):
+    """The last limb count of the small-launch tile at logN = 16 and 17, per pass."""
+    def last(kind, logN, operands=False):
+        got = variant(kind, logN, range(1, 201), operands, fold=fold)
+        return got.index(next(v for v in got if v != 5)) if set(got) != {5} else None
+
+    assert [last(k, 16) for k in range(4)] == [22, 28 if fold else 32, 32, 23]
+    assert [last(k, 17) for k in range(4)] == [11, 14 if fold else 16, 16, 11]
+    assert last(FWD_ROWS, 16, True) == (56 if fold else None)
 
 
 @pytest.mark.parametrize("logN", [13, 14, 15, 16, 17])
