@@ -66,11 +66,11 @@ constexpr int ntt_compiled(int v, bool fold, int kind)
 //     logN = 17, 20: 32.9 32.2, 60: 94.4 90.4.  Shoup, 30: 27.5 27.7, 36: 31.4 30.8
 // Large row passes take four rows a CTA, at logN = 13 eight: four rows of 64
 // elements are half a warp (480 limbs forward 43.4 us with four, 32.1 with eight).
-// Forward columns run within 64 registers at logN = 17 past 12 limbs (80 against
-// 64: 12 limbs 20.5 20.7, 15: 25.2 24.7, 30: 43.4 43.2, 60: 85.0 83.9, 90: 125.8
-// 123.5; not at logN = 16: 60 limbs 35.4 35.7, 180: 106.3 107.3), with Shoup
-// products past 44 of logN = 16 (30: 25.9 26.3, 60: 43.8 42.8, 90: 65.3 63.8; logN =
-// 15, 60: 24.3 25.5, 90: 32.9 32.5).
+// Forward columns run within 64 registers past 64 limbs of logN = 17 with folding
+// products (80 against 64: 90 limbs 125.8 123.5, 120: 165.0 162.0; logN = 16, 180
+// limbs 106.3 107.3).  Plain transforms of 15 to 60 limbs of logN = 17 gain 1 % by
+// it too, but the columns of a Rescale, which reduce their input, lose more (14
+// limbs 31.9 35.7), and so with Shoup products.
 //
 // operands: a forward row pass whose epilogue reads operands (ModDown,
 // Rescale: two or three words a coefficient against one) waits for HBM where
@@ -88,7 +88,7 @@ inline int ntt_default_variant(int kind, int logN, bool fold, long total, bool o
     const long limbs = ((total << logN) + 65535) >> 16;   // of logN = 16, rounded up
     const int rows16 = logN == 13 ? 1 : 2;                // row passes with sixteen elements
     switch (kind) {
-    case FWD_COLS: return limbs <= 22 ? 5 : (limbs > (logN == 17 ? 24 : 44) && (logN == 17 || !fold) ? 4 : 1);
+    case FWD_COLS: return limbs <= 22 ? 5 : (logN == 17 && fold && limbs > 128 ? 4 : 1);
     case INV_COLS: return limbs <= 23 ? 5 : 1;
     case FWD_ROWS:
         if (operands) return !fold || limbs <= 56 ? 5 : (logN == 13 ? 4 : 3);
