@@ -160,13 +160,16 @@ int fides_ctx_add_stream(fides_ctx *ctx, void *stream);
  * per GPU; every launch here covers all limbs of a step, and what is tuned is
  * the tile width of each pass, which sets the CTA count and hence how full the
  * last wave is).  Times each tile variant (16, 8 or 4 columns or rows per CTA,
- * with a 64- or 80-register budget, 16 or 8 elements per thread) of each
- * two-pass transform's pass for every limb count 1..max_limbs (at most 128; larger
- * launches use the choice for 128) on this context's scratch, and keeps the
- * fastest; forward rows are timed with a plain epilogue and with one that reads
- * operands (ModDown, Rescale), together, since one choice serves both.  Without it the variant goes by the launch's size, whatever its limb
- * count.  Results are unchanged by the choice.  Synchronises `stream`; do not run it while other work uses
- * this context.  logN = 12 has a single variant (returns FIDES_OK at once).
+ * with a 64- or 80-register budget, 16 or 8 elements per thread) of each pass of
+ * a two-pass transform for every limb count 1..max_limbs (at most 128; larger
+ * launches use the choice for 128) on this context's scratch.  A variant that is
+ * faster than the default, in a transform by itself and in a chain of them,
+ * replaces it (about 1.5 s for 128 limbs of logN = 16).  Forward rows are timed
+ * with a plain epilogue and with one that reads operands (ModDown, Rescale),
+ * together, since one choice serves both.  Without it the variant goes by the
+ * launch's size, whatever its limb count.  Results are unchanged by the choice.
+ * Synchronises `stream`; do not run it while other work uses this context.
+ * logN = 12 has a single variant (returns FIDES_OK at once).
  * fides_ctx_ntt_tile reports the tile that runs for pass 0..3 (forward
  * columns, forward rows with a plain epilogue, inverse rows, inverse columns) at
  * n_limbs as (tile width << 8) | resident CTAs per SM, the latter the target

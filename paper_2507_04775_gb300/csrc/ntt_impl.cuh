@@ -162,26 +162,24 @@ int rows_inner(const fides_ctx *c, const IPArgs &A, int limbs, int max_beta, cud
     return fides_set_error(FIDES_ERR_UNSUPPORTED, "rows + inner product: logN = 12");   // rows_inner_ok is false
 }
 
-// One pass of kind `kind` with variant v (for the autotuner).  Forward rows run
-// twice, once with an epilogue that reads operands (the segments carry aux, out
-// and constants): one choice serves both.
+// What the autotuner times for variant v of pass kind `kind`: whole transforms,
+// whose other pass runs the default tile.  Forward rows run twice, once with an
+// epilogue that reads operands (the segments carry aux, out and constants): one
+// choice serves both.
 template <int LOGN>
 void launch_one(const fides_ctx *c, int kind, int v, const LimbSet &set, cudaStream_t st)
 {
-    switch (kind) {
-    case FWD_COLS:
-        launch_pass_v<LOGN, 0, false, false>(v, c, set, c->d_tw, ProSrc{}, EpiLazy{}, st, "k_ntt_tune");
-        break;
-    case FWD_ROWS:
-        launch_pass_v<LOGN, 1, false, false>(v, c, set, c->d_tw, ProDst{}, EpiCanon{}, st, "k_ntt_tune");
-        launch_pass_v<LOGN, 1, false, false>(v, c, set, c->d_tw, ProDst{}, EpiSubMul{}, st, "k_ntt_tune");
-        break;
-    case INV_ROWS:
-        launch_pass_v<LOGN, 1, true, false>(v, c, set, c->d_itw, ProPlain{}, EpiLazy{}, st, "k_ntt_tune");
-        break;
-    default:
-        launch_pass_v<LOGN, 0, true, true>(v, c, set, c->d_itw, ProDst{}, EpiCanon{}, st, "k_ntt_tune");
-        break;
+    const char *name = "k_ntt_tune";
+    auto tile = [&](int k) { return k == kind ? v : ntt_default_variant(k, LOGN, c->fold, set.total); };
+    if (kind == FWD_COLS || kind == FWD_ROWS) {
+        launch_pass_v<LOGN, 0, false, false>(tile(FWD_COLS), c, set, c->d_tw, ProSrc{}, EpiLazy{}, st, name);
+        launch_pass_v<LOGN, 1, false, false>(tile(FWD_ROWS), c, set, c->d_tw, ProDst{}, EpiCanon{}, st, name);
+        if (kind == FWD_COLS) return;
+        launch_pass_v<LOGN, 0, false, false>(tile(FWD_COLS), c, set, c->d_tw, ProSrc{}, EpiLazy{}, st, name);
+        launch_pass_v<LOGN, 1, false, false>(v, c, set, c->d_tw, ProDst{}, EpiSubMul{}, st, name);
+    } else {
+        launch_pass_v<LOGN, 1, true, false>(tile(INV_ROWS), c, set, c->d_itw, ProPlain{}, EpiLazy{}, st, name);
+        launch_pass_v<LOGN, 0, true, true>(tile(INV_COLS), c, set, c->d_itw, ProDst{}, EpiCanon{}, st, name);
     }
 }
 

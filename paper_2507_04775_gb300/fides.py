@@ -370,7 +370,7 @@ class Context:
         return int(lib().fides_galois_elt(self._h, steps))
 
     def autotune(self, max_limbs: int = 128, stream=None, cache: str | None = None):
-        """Time the NTT tile variants per pass and limb count; keep the fastest.
+        """Time the NTT tile variants per pass and limb count; keep those that beat the default.
         With `cache`, a table tuned earlier for the same device and parameters
         is loaded from that JSON file instead, and a new one is saved there."""
         key = None
