@@ -377,8 +377,9 @@ class Context:
         if cache:
             import json
             import torch
+            # (the primes decide which arithmetic, and so which kernels, run)
             key = {"device": torch.cuda.get_device_name(), "logN": self.logN, "L": self.L, "K": self.K,
-                   "library": version()}
+                   "primes": self.q + self.p, "library": version()}
             try:
                 entry = json.load(open(cache))
                 if entry.get("key") == key:
