@@ -166,7 +166,8 @@ int fides_ctx_add_stream(fides_ctx *ctx, void *stream);
  * faster than the default, in a transform by itself and in a chain of them,
  * replaces it (about 1.5 s for 128 limbs of logN = 16).  Forward rows are timed
  * with a plain epilogue and with one that reads operands (ModDown, Rescale),
- * together, since one choice serves both.  Without it the variant goes by the
+ * together, since one choice serves both (the default has one for each).
+ * Without it the variant goes by the
  * launch's size, whatever its limb count.  Results are unchanged by the choice.
  * Synchronises `stream`; do not run it while other work uses this context.
  * logN = 12 has a single variant (returns FIDES_OK at once).
@@ -184,8 +185,10 @@ int fides_ctx_ntt_tile(const fides_ctx *ctx, int pass, int n_limbs);
  * The tuned table itself, for an autotuner cache: FIDES_TUNE_ENTRIES bytes,
  * the variant index per pass kind (4) and limb count (0..128).  set = 0
  * copies the context's table out; set = 1 installs `table` (FIDES_ERR_ARG,
- * nothing changed, if an entry is not a variant index).  Installing the table
- * that an untuned context gives out restores the choice by size.
+ * nothing changed, if an entry is not a variant index).  An entry equal to the
+ * default's leaves the default, which may run forward rows whose epilogue reads
+ * operands in a tile of their own; any other entry decides both.  Installing the
+ * table that an untuned context gives out restores the choice by size.
  */
 #define FIDES_TUNE_ENTRIES (4 * 129)
 int fides_ctx_tune_table(fides_ctx *ctx, unsigned char *table, int set);

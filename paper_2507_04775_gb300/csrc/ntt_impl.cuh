@@ -165,7 +165,7 @@ int rows_inner(const fides_ctx *c, const IPArgs &A, int limbs, int max_beta, cud
 // What the autotuner times for variant v of pass kind `kind`: whole transforms,
 // whose other pass runs the default tile.  Forward rows run twice, once with an
 // epilogue that reads operands (the segments carry aux, out and constants): one
-// choice serves both.
+// choice serves both, the default with its own tile for the latter.
 template <int LOGN>
 void launch_one(const fides_ctx *c, int kind, int v, const LimbSet &set, cudaStream_t st)
 {
@@ -176,7 +176,9 @@ void launch_one(const fides_ctx *c, int kind, int v, const LimbSet &set, cudaStr
         launch_pass_v<LOGN, 1, false, false>(tile(FWD_ROWS), c, set, c->d_tw, ProDst{}, EpiCanon{}, st, name);
         if (kind == FWD_COLS) return;
         launch_pass_v<LOGN, 0, false, false>(tile(FWD_COLS), c, set, c->d_tw, ProSrc{}, EpiLazy{}, st, name);
-        launch_pass_v<LOGN, 1, false, false>(v, c, set, c->d_tw, ProDst{}, EpiSubMul{}, st, name);
+        const int def = ntt_default_variant(FWD_ROWS, LOGN, c->fold, set.total);
+        launch_pass_v<LOGN, 1, false, false>(v == def ? ntt_default_variant(FWD_ROWS, LOGN, c->fold, set.total, true) : v,
+                                             c, set, c->d_tw, ProDst{}, EpiSubMul{}, st, name);
     } else {
         launch_pass_v<LOGN, 1, true, false>(tile(INV_ROWS), c, set, c->d_itw, ProPlain{}, EpiLazy{}, st, name);
         launch_pass_v<LOGN, 0, true, true>(tile(INV_COLS), c, set, c->d_itw, ProDst{}, EpiCanon{}, st, name);

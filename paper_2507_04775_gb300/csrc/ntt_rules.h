@@ -97,12 +97,15 @@ inline int ntt_default_variant(int kind, int logN, bool fold, long total, bool o
     }
 }
 
-// Variant of a pass: what the tuned or installed table (n entries for the pass
-// kind, limb counts from zero) says, whatever the epilogue, or the default.
-// Launches past the table's end take its last entry.
+// Variant of a pass: what the tuned or installed table says (n entries for the
+// pass kind, limb counts from zero; launches past its end take the last), or
+// the default.  An entry that is the default's leaves the default, also for the
+// passes whose epilogue reads operands; any other is what runs in both.
 inline int ntt_variant(const unsigned char *table, int n, bool tuned, int kind, int logN, bool fold, int total,
                        bool operands)
 {
-    if (!tuned) return ntt_default_variant(kind, logN, fold, total, operands);
-    return table[total < n ? total : n - 1];
+    const int at = total < n ? total : n - 1;
+    if (!tuned || (operands && table[at] == ntt_default_variant(kind, logN, fold, at)))
+        return ntt_default_variant(kind, logN, fold, total, operands);
+    return table[at];
 }

@@ -78,8 +78,12 @@ def test_lines(variant, fold):
 @pytest.mark.parametrize("logN", [13, 14, 15, 16, 17])
 def test_an_installed_table_decides_every_pass(variant, logN):
     """Every entry is what runs, with and without an epilogue that reads
-    operands, and the last one past the table's end."""
+    operands, and the last one past the table's end; an entry equal to the
+    default's leaves the default."""
     for kind in range(4):
+        plain, own = variant(kind, logN, range(0, 300)), variant(kind, logN, range(0, 300), True)
         for operands in (False, True):
             got = variant(kind, logN, range(0, 300), operands, tuned=True)
-            assert got == [min(i, 128) % 6 for i in range(300)]
+            for i, v in enumerate(got):
+                entry = min(i, 128) % 6
+                assert v == (own[i] if operands and entry == plain[min(i, 128)] else entry)
