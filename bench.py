@@ -306,9 +306,10 @@ LANE_CYCLES_PER_MODMUL = 10
 FMAHEAVY_LANES_PER_CLK_SM = 64
 SMS = 152
 
-# What limits each kernel, from its ncu profile: the NTT passes the integer
-# multiply pipe, the inner and tensor products DRAM, the conversion the
-# tensor-core issue path.
+# What limits each kernel, from its ncu profile (profiles/hmult_kernels_logN16_L30.md,
+# profiles/ops_kernels_logN16_L30.md): the NTT passes the integer multiply pipe
+# and their own chains, the plain inner product, the tensor product and the
+# element-wise kernels DRAM, the conversion the tensor-core issue path.
 KERNEL_BOUND = {"k_ntt": "alu", "k_rows_inner": "alu", "k_inner": "hbm", "k_tensor": "hbm", "k_elem": "hbm", "k_ptmac": "hbm",
                 "k_bconv_tc": "tensor"}
 
@@ -1185,10 +1186,11 @@ def load_traffic(kernel, bytes_per_launch):
     return int(ent["dram_bytes_per_unit"] * bytes_per_launch / ent["algorithmic_bytes_per_unit"])
 
 
-KERNEL_SOURCES = {"k_ntt": ["ntt.cuh", "ntt_impl.cuh", "ntt_l16.cu", "fides_internal.cuh"],
+KERNEL_SOURCES = {"k_ntt": ["ntt.cuh", "ntt_impl.cuh", "ntt_rules.h", "ntt_l16.cu", "fides_internal.cuh"],
                   "k_bconv_tc": ["bconv_tc.cuh", "kernels.cuh", "fides_internal.cuh"],
                   "k_bconv": ["kernels.cuh", "fides_internal.cuh"],
-                  "k_rows_inner": ["rows_inner.cuh", "ntt.cuh", "ntt_impl.cuh", "ntt_l16.cu", "fides_internal.cuh"],
+                  "k_rows_inner": ["rows_inner.cuh", "ntt.cuh", "ntt_impl.cuh", "ntt_rules.h", "ntt_l16.cu",
+                                   "fides_internal.cuh"],
                   "k_inner": ["kernels.cuh", "rows_inner.cuh", "fides_internal.cuh"]}
 
 

@@ -252,8 +252,10 @@ int fides_ctx_rounding(const fides_ctx *ctx);
 
 /*
  * Whether base conversions of this context run on the tensor cores (1: every
- * digit and K have at most 16 primes) or on the integer pipes (0).  Results
- * are identical.
+ * digit and K have at most 16 primes) or some on the integer pipes (0).
+ * Launches so small that the integer kernel is faster go there in either case
+ * (at most 16 targets and 2^21 products, ten and 2^22 or six and 2^24; eight
+ * targets at logN = 12).  Results are identical.
  */
 int fides_ctx_tensor_bconv(const fides_ctx *ctx);
 

@@ -6,14 +6,15 @@
 // to tune is the tile width of each pass, which decides how many CTAs a launch
 // has and so how much of its last wave is empty, and the elements per thread.
 // Six variants of each pass of a two-pass transform (logN 13..17) are compiled
-// -- at logN=16, sixteen elements per thread with 16, 8 or 4 columns/rows per
+// for folding products (three or four for Shoup products, ntt_compiled) -- at
+// logN=16, sixteen elements per thread with 16, 8 or 4 columns/rows per
 // CTA (256, 128 or 64 threads) and up to 80 registers (3, 6 or 12 resident
 // CTAs per SM), or with 4 or 8 per CTA and up to 64 registers (16 or 8 per
 // SM), and eight elements per thread with 4 per CTA (128 threads, 8 per SM, 64
 // registers); other sizes scale the resident-CTA target to the same register
-// budget (ntt_impl.cuh) -- and the context keeps, per pass kind and limb
-// count, the variant to launch: a default by size, or the fastest measured one
-// after fides_ctx_autotune.  The launchers of each ring degree live in
+// budget (ntt_rules.h).  The variant of a launch is a default by its size, or
+// after fides_ctx_autotune what a table of the context says per pass kind and
+// limb count.  The launchers of each ring degree live in
 // ntt_l12.cu .. ntt_l17.cu; this file dispatches on the context's logN.
 #include <algorithm>
 #include <cstring>

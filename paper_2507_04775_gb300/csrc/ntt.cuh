@@ -17,8 +17,8 @@
 //     contiguous rows (S_col, S_row = 7+6, 7+7, 8+7, 8+8, 9+8 for logN 13..17).
 //     Four global accesses per element, as in the paper.  CT is 16, 8 or 4;
 //     narrower tiles split a small launch into more CTAs so its last wave
-//     costs less (the choice per pass and limb count is autotuned, see
-//     ntt.cu).
+//     costs less (the choice per pass goes by the launch's size or by a tuned
+//     table, see ntt_rules.h).
 // Inside a pass, stages are grouped LE at a time ("rounds"): in a round every
 // thread owns 2^LE elements whose local indices differ only in the round's LE
 // bits, so LE radix-2 stages run in registers (a pass whose stage count is

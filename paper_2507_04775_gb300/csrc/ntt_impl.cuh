@@ -8,9 +8,9 @@
 //   logN   13   14   15   16   17
 //   S_col   7    7    8    8    9
 //   S_row   6    7    7    8    8
-// Each pass has six compiled tile variants (columns/rows per CTA, the
+// Each pass has up to six compiled tile variants (columns/rows per CTA, the
 // resident-CTA target and the elements per thread, chosen per pass kind and
-// limb count; see ntt.cu).
+// size; see ntt_rules.h).
 #pragma once
 
 #include <algorithm>

@@ -15,12 +15,13 @@
 // What it replaces at logN = 16, 30 limbs, three digits: the row pass of 90
 // limbs (33 us by itself), the inner product (HBM bound on 189 MB, of which 47 MB
 // are the digits re-read, 37 us) and the inverse row pass of 20 limbs (13 us).
-// It takes 76 us, bound by the latency of its own chain at 24 warps per SM (46 %
+// It takes 74 us, bound by the latency of its own chain at 22 warps per SM (45 %
 // of issue slots), and two launches fewer; the key words of a tile are on their
 // way to L2 while the digits transform.  HMult at logN = 16: 10 limbs 106.6 ->
 // 98.5 us, 17: 144.8 -> 139.4, 30: 235.0 -> 233.0; logN = 17, 36 limbs, four
-// digits: 652.9 -> 627.7.  More CTAs per SM lose to the L1 their tiles take
-// (four digits: 197 us with five, 207 with six, 243 with seven).
+// digits: 652.9 -> 627.7.  Six CTAs per SM up to three digits, five above: more
+// lose to the L1 their tiles take (four digits: 197 us with five, 207 with six,
+// 243 with seven).
 #pragma once
 
 #include "fides_internal.cuh"

@@ -360,7 +360,7 @@ class Context:
 
     @property
     def tensor_bconv(self) -> bool:
-        """Whether base conversions run on the tensor cores."""
+        """Whether base conversions run on the tensor cores (but for launches small enough for the integer kernel)."""
         return bool(lib().fides_ctx_tensor_bconv(self._h))
 
     def psi(self, i: int) -> int:
